@@ -321,6 +321,8 @@ void set_reciprocals(Level& L) {
   for (int q = 0; q < 7; ++q) {
     const double cd = (double)d2 + L.alpha * q + L.sh2;
     const float cf = (float)d2 + L.alphaf * (float)q + L.sh2f;
+    L.cf[q] = cf;
+    L.cd[q] = cd;
     L.rcd[q] = cd > 0 ? 1.0 / cd : 0.0;
     L.rcf[q] = cf > 0 ? 1.0f / cf : 0.0f;
     L.cdh[q] = (float)cd;
@@ -560,12 +562,38 @@ bool run_lower_cycle(vsv_grid* g, const std::vector<Level>& lv, int l, Comp3<T> 
   return launch_lower_vcycle<T>(g->cx, P);
 }
 
+// Largest level of the two-sweep passes: their halo makes them do each
+// half-sweep 2 to 5 times over, which the launches they save pay for up to
+// here (128 x 64 x 64: 24 + 39 us against 32 + 31 us of fused sweeps and tiled
+// transfers; 64 x 32 x 32: 7 + 10 us against 27 + 25 us level by level).
+const long long kPassCells = 1LL << 18;
+// Largest finest level whose pre-smoothing pass also restricts its residual
+// (a solve at 64 x 32 x 32: 652 -> 639 us); above, the tiled restriction.
+const long long kPassFineRestrict = 1LL << 17;
+
+// Do the two-sweep passes (passes.cu) run this level's smoothing?  V(2,2)
+// cycles of variant 0 from e = 0 on levels they serve; not while a kernel
+// class is being profiled (a pass belongs to several classes, the separate
+// kernels to one each; the results are the same bits).
+template <class T>
+bool passes_wanted(const vsv_grid* g, const std::vector<Level>& lv, int l, bool x_zero,
+                   const Rhs3<T>& R) {
+  if (!std::is_same<T, float>::value || g->prec != VSV_MIXED) return false;
+  if (lv[l].cells() > kPassCells) return false;
+  return g->sol.variant == 0 && g->sol.nu1 == 2 && g->sol.nu2 == 2 && x_zero && R.beta == (T)1 &&
+         !R.S[0] && !R.S[1] && !R.S[2] && g->cx.prof_class < 0 && l + 1 < (int)lv.size() &&
+         two_sweep_pass_ok(lv[l], lv[l + 1]);
+}
+
 // One V-cycle from level l for L x = R.  uh / ul as in smooth(): returns
 // true if the correction was added to that iterate by the last sweep.
+// *where: the buffer that holds the result otherwise (X, or the level's
+// ping-pong partner after a post-smoothing pass).
 template <class T>
 bool vcycle(vsv_grid* g, const std::vector<Level>& lv, int l, Comp3<T> X, Rhs3<T> R, int ncomp,
             bool exact_fine = true, bool x_zero = false, const Comp3<float>* uh = nullptr,
-            const Comp3<float>* ul = nullptr) {
+            const Comp3<float>* ul = nullptr, Comp3<T>* where = nullptr) {
+  if (where) *where = X;
   const Level& L = lv[l];
   const double h2 = 1.0 / L.inv_h2;
   const bool last = (l + 1 == (int)lv.size());
@@ -601,14 +629,32 @@ bool vcycle(vsv_grid* g, const std::vector<Level>& lv, int l, Comp3<T> X, Rhs3<T
     Comp3<T> RR{{(T*)R.B[0], (T*)R.B[1], (T*)R.B[2]}};
     if (launch_coarse_vcycle<T>(g->cx, CC, X, RR, ncomp)) return false;
   }
-  smooth<T>(g, L, l, X, R, ncomp, g->sol.nu1, x_zero);
   const Level& C = lv[l + 1];
   Comp3<T> EC = cview<T>(g->mg_e[l + 1], g->c0);
   Comp3<T> RC = cview<T>(g->mg_r[l + 1], g->c0);
+  if constexpr (std::is_same<T, float>::value) {
+    if ((uh && ul) || where) {
+      if (passes_wanted<T>(g, lv, l, x_zero, R)) {
+        const float w = (float)mg_weight(g);
+        const Comp3<float> RR{{(float*)R.B[0], (float*)R.B[1], (float*)R.B[2]}};
+        const bool rst = l > 0 || L.cells() <= kPassFineRestrict;
+        launch_pre_pass(g->cx, L, C, RR, X, RC, ncomp, w, rst, kc);
+        if (!rst) launch_resid_restrict<T>(g->cx, L, C, X, R, RC, ncomp, false);
+        Rhs3<T> RCr{{RC.p[0], RC.p[1], RC.p[2]}, {nullptr, nullptr, nullptr}, (T)1};
+        vcycle<T>(g, lv, l + 1, EC, RCr, ncomp, exact_fine, true, nullptr, nullptr, &EC);
+        Comp3<float> out = cview<float>(g->mg_t[l], g->c0);
+        launch_post_pass(g->cx, L, C, RR, X, EC, out, uh, ul, ncomp, w, kc);
+        if (uh && ul) return true;
+        *where = out;
+        return false;
+      }
+    }
+  }
+  smooth<T>(g, L, l, X, R, ncomp, g->sol.nu1, x_zero);
   const bool exact = std::is_same<T, float>::value && l == 0 && exact_fine;
   launch_resid_restrict<T>(g->cx, L, C, X, R, RC, ncomp, exact);
   Rhs3<T> RCr{{RC.p[0], RC.p[1], RC.p[2]}, {nullptr, nullptr, nullptr}, (T)1};
-  vcycle<T>(g, lv, l + 1, EC, RCr, ncomp, exact_fine, true);
+  vcycle<T>(g, lv, l + 1, EC, RCr, ncomp, exact_fine, true, nullptr, nullptr, &EC);
   launch_prolong_add<T>(g->cx, L, C, X, EC, ncomp);
   return smooth<T>(g, L, l, X, R, ncomp, g->sol.nu2, false, uh, ul);
 }

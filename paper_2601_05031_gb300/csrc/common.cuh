@@ -33,6 +33,12 @@ struct Level {
   // sweep kernel)
   float rcf[7];
   double rcd[7];
+  // the diagonal coefficient 2 d + alpha * nwall + sh2 itself, rounded to
+  // each type: every residual kernel reads it instead of forming it per cell
+  // (on the FP64 path a conversion, an FMA and an addition on units that do
+  // two operations per clock and SM)
+  float cf[7];
+  double cd[7];
   // the diagonal coefficient 2 d + alpha * nwall + sh2 as an FP32 pair
   // (hi + lo) for the exact defect
   float cdh[7], cdl[7];
@@ -42,6 +48,10 @@ struct Level {
 template <class T> __host__ __device__ inline T lv_rc(const Level& L, int nwall);
 template <> __host__ __device__ inline float lv_rc<float>(const Level& L, int nwall) { return L.rcf[nwall]; }
 template <> __host__ __device__ inline double lv_rc<double>(const Level& L, int nwall) { return L.rcd[nwall]; }
+
+template <class T> __host__ __device__ inline T lv_coef(const Level& L, int nwall);
+template <> __host__ __device__ inline float lv_coef<float>(const Level& L, int nwall) { return L.cf[nwall]; }
+template <> __host__ __device__ inline double lv_coef<double>(const Level& L, int nwall) { return L.cd[nwall]; }
 
 template <class T> __host__ __device__ inline T lv_alpha(const Level& L);
 template <> __host__ __device__ inline float lv_alpha<float>(const Level& L) { return L.alphaf; }
@@ -64,6 +74,20 @@ struct Comp3 {
   }
 };
 
+// Correctly rounded a b + c and a b in T, never contracted or split by the
+// compiler: the kernels that must agree bit for bit share formulas written
+// with these.
+template <class T>
+__device__ __forceinline__ T fma_t(T a, T b, T c) {
+  if constexpr (sizeof(T) == 4) return __fmaf_rn(a, b, c);
+  else return __fma_rn(a, b, c);
+}
+template <class T>
+__device__ __forceinline__ T mul_t(T a, T b) {
+  if constexpr (sizeof(T) == 4) return __fmul_rn(a, b);
+  else return __dmul_rn(a, b);
+}
+
 // Prolongation increment of one fine cell (cell-centred trilinear, weights
 // 3/4 and 1/4 per axis).  The arguments are the (x-centre, x-neighbour) pairs
 // of coarse values, already multiplied by their boundary factors, for the
@@ -71,14 +95,22 @@ struct Comp3 {
 // plane, centre row) and (neighbour plane, neighbour row).  Every
 // prolongation kernel calls this, so they agree bit for bit.
 template <class T>
+__device__ __forceinline__ T prolong_pair(T c, T x) {   // 3/4 c + 1/4 x
+  return fma_t((T)0.75, c, mul_t((T)0.25, x));
+}
+template <class T>
 __device__ __forceinline__ T prolong_value(T aC, T aX, T bC, T bX, T cC, T cX, T dC, T dX) {
-  const T w1 = (T)0.75, w2 = (T)0.25;
-  T acc = 0;
-  acc += w1 * w1 * (w1 * aC + w2 * aX);
-  acc += w1 * w2 * (w1 * bC + w2 * bX);
-  acc += w2 * w1 * (w1 * cC + w2 * cX);
-  acc += w2 * w2 * (w1 * dC + w2 * dX);
-  return acc;
+  T acc = mul_t((T)0.5625, prolong_pair(aC, aX));
+  acc = fma_t((T)0.1875, prolong_pair(bC, bX), acc);
+  acc = fma_t((T)0.1875, prolong_pair(cC, cX), acc);
+  return fma_t((T)0.0625, prolong_pair(dC, dX), acc);
+}
+
+// b - L x of one cell: (neighbour sum s) - coef x, times 1 / h^2, from b;
+// shared by every residual and restriction kernel.
+template <class T>
+__device__ __forceinline__ T resid_value(T b, T s, T coef, T x, T ih2) {
+  return fma_t(-fma_t(-coef, x, s), ih2, b);
 }
 
 // Weighted red-black update of one cell (red-black SOR smoothing; an

@@ -249,6 +249,17 @@ void launch_rbgs_fused(Ctx& cx, const Level& L, Comp3<float> A, Comp3<float> B, 
 bool launch_copy_wait_probe(Ctx& cx, const Level& L, Comp3<float> B, Rhs3<float> R,
                             unsigned probe_tx, unsigned long long limit_ns);
 
+// two-sweep passes of a V-cycle (passes.cu): a level's whole pre-smoothing
+// from e = 0 (restrict_: and its residual on the next level), its whole
+// post-smoothing (prolongation included; the result added to the iterate
+// upd_hi / upd_lo, or stored to OUT, which must not be E)
+bool two_sweep_pass_ok(const Level& F, const Level& C);
+void launch_pre_pass(Ctx& cx, const Level& F, const Level& C, Comp3<float> R, Comp3<float> E,
+                     Comp3<float> RC, int ncomp, float omega, bool restrict_, int kclass);
+void launch_post_pass(Ctx& cx, const Level& F, const Level& C, Comp3<float> R, Comp3<float> E,
+                      Comp3<float> EC, Comp3<float> OUT, const Comp3<float>* upd_hi,
+                      const Comp3<float>* upd_lo, int ncomp, float omega, int kclass);
+
 // ---------------------------------------------------------------- phase-field (phase.cu)
 struct PhaseParams {
   int nx, ny, nz, zper;

@@ -71,8 +71,6 @@ __device__ __forceinline__ T rhs_at(const Rhs3<T>& R, int comp, long long c, int
   return b;
 }
 
-__device__ __forceinline__ int n_active(const Level& L) { return L.act[0] + L.act[1] + L.act[2]; }
-
 // ---------------------------------------------------------------- residual value
 // r = b - L_h x at one cell, plain arithmetic in T.
 template <class T>
@@ -80,8 +78,7 @@ __device__ __forceinline__ T resid_plain(const T* __restrict__ x, const Level& L
                                          long long c, T b) {
   int nwall;
   const T s = sum_nb(x, L, i, j, k, c, nwall);
-  T coef = (T)(2 * n_active(L)) + lv_alpha<T>(L) * (T)nwall + lv_sh2<T>(L);
-  return b - (s - coef * x[c]) * lv_ih2<T>(L);
+  return resid_value(b, s, lv_coef<T>(L, nwall), x[c], lv_ih2<T>(L));
 }
 
 // Exact defect in FP32 storage: every term of b - (sum_nb - coef x_c)/h^2 is
@@ -411,7 +408,7 @@ __global__ void k_restrict_block(Level F, Level C, Comp3<T> X, Rhs3<T> R, Comp3<
     if (zm >= 0) ld2(row(j0 + jy, zm) + i0, fzm[jy][0], fzm[jy][1]); else fzm[jy][0] = fzm[jy][1] = (T)0;
     if (zp >= 0) ld2(row(j0 + jy, zp) + i0, fzp[jy][0], fzp[jy][1]); else fzp[jy][0] = fzp[jy][1] = (T)0;
   }
-  const T ih2 = lv_ih2<T>(F), al = lv_alpha<T>(F), sh = lv_sh2<T>(F);
+  const T ih2 = lv_ih2<T>(F);
   T acc = 0;
 #pragma unroll
   for (int kz = 0; kz < 2; ++kz)
@@ -428,7 +425,7 @@ __global__ void k_restrict_block(Level F, Level C, Comp3<T> X, Rhs3<T> R, Comp3<
         const int nwall = (ix == 0 && xm < 0) + (ix == 1 && xp < 0) + (jy == 0 && ym < 0) +
                           (jy == 1 && yp < 0) + (kz == 0 && zm < 0) + (kz == 1 && zp < 0);
         const T s = ((v_xm + v_xp) + (v_ym + v_yp)) + (v_zm + v_zp);
-        acc += b[kz][jy][ix] - (s - ((T)6 + al * (T)nwall + sh) * c[kz][jy][ix]) * ih2;
+        acc += resid_value(b[kz][jy][ix], s, lv_coef<T>(F, nwall), c[kz][jy][ix], ih2);
       }
   RC.at(comp)[lin(I, J, K, C.n[0], C.n[1])] = acc * (T)0.125;
 }

@@ -18,7 +18,8 @@ constexpr int kRS = 5;         // ring slots
 constexpr int kRStage = (kRR * kNV + kThreads - 1) / kThreads;
 
 struct RGeom : Geom {
-  float ih2, alpha, beta, sh2;
+  float ih2, beta;
+  float cf0, cf1, cf2;   // diagonal coefficient with 0, 1, 2 wall neighbours
   int cnx, cny;   // coarse extents (x, y)
 };
 
@@ -118,13 +119,14 @@ k_restrict_tiled(RGeom G, Comp3<float> X, Rhs3<float> R, Comp3<float> RC) {
       const float Lx = row[4 * q - 1], Rx = row[4 * q + 4];
       const float s_ = (HAS_S && act) ? S[jown[h] + (long long)p * G.ny] : 0.f;
       const int nwall = yw[h] + zw;
+      const float coef = nwall == 0 ? G.cf0 : (nwall == 1 ? G.cf1 : G.cf2);
 #pragma unroll
       for (int o = 0; o < 4; ++o) {
         const float xm = o == 0 ? Lx : c4(Vz[h], o - 1);
         const float xp = o == 3 ? Rx : c4(Vz[h], o + 1);
         const float s = ((xm + xp) + (c4(U, o) + c4(D, o))) + (c4(Mz[h], o) + c4(Pz[h], o));
         const float b = G.beta * c4(Bc[h], o) + s_;
-        const float r = b - (s - (6.f + G.alpha * (float)nwall + G.sh2) * c4(Vz[h], o)) * G.ih2;
+        const float r = resid_value(b, s, coef, c4(Vz[h], o), G.ih2);
         if (o < 2) acc0 += r; else acc1 += r;
       }
     }
@@ -313,8 +315,9 @@ bool launch_restrict_tiled(Ctx& cx, const Level& F, const Level& C, Comp3<float>
   RGeom G;
   static_cast<Geom&>(G) = geom(F, even_chunk(F, std::max(ncomp, cx.chunk_comps), cx.sms, 2));
   G.ih2 = F.inv_h2f;
-  G.alpha = F.alphaf;
-  G.sh2 = F.sh2f;
+  G.cf0 = F.cf[0];
+  G.cf1 = F.cf[1];
+  G.cf2 = F.cf[2];
   G.beta = R.beta;
   G.cnx = C.n[0];
   G.cny = C.n[1];

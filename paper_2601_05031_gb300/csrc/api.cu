@@ -510,8 +510,28 @@ bool coarse_plan(const vsv_grid* g, const std::vector<Level>& lv, int m, CoarseC
     CC->lv[q] = lv[q];
     CC->h2[q] = 1.0 / lv[q].inv_h2;
     CC->off[q] = off;
-    off += 2 * lv[q].cells();
+    // e and r of the two colours, each of half a row's length rounded up
+    const long long cols = (long long)((lv[q].n[0] + 1) / 2) * lv[q].n[1], nz = lv[q].n[2];
+    off += 4LL * cols * nz;
+    // the shortest runs along z whose threads fit; on a level that runs of 1 to
+    // 8 (FP64: 4) planes do not cover evenly, as many threads as there are
+    const long long n = std::min<long long>(kCvThreads, (cols * nz + 31) / 32 * 32);
+    long long len = 0;
+    for (long long t = 1; t <= (elem == 4 ? 8 : 4) && !len; t *= 2)
+      if (nz % t == 0 && cols * (nz / t) <= n) len = t;
+    CC->reg[q] = len > 0;
+    if (!len) {
+      const long long segs = std::max(1LL, n / cols);
+      len = (nz + segs - 1) / segs;
+    }
+    CC->run[q] = (int)len;
+    CC->runs[q] = (int)std::min<long long>(cols * ((nz + len - 1) / len), 1 << 30);
+    CC->threads[q] = CC->reg[q] ? (CC->runs[q] + 31) / 32 * 32 : (int)n;
   }
+  // a level's threads include those of the levels below it
+  for (int q = CC->last; q > m; --q) CC->threads[q - 1] = std::max(CC->threads[q - 1], CC->threads[q]);
+  CC->scratch = (int)std::min<long long>(off, 1 << 30);   // residuals, one value per cell of level m
+  off += 2LL * ((lv[m].n[0] + 1) / 2) * lv[m].n[1] * lv[m].n[2];
   CC->total = off;
   return (size_t)off * elem <= kCoarseCycleSmem;
 }
@@ -585,6 +605,13 @@ bool passes_wanted(const vsv_grid* g, const std::vector<Level>& lv, int l, bool 
          two_sweep_pass_ok(lv[l], lv[l + 1]);
 }
 
+// Largest first level of the one-CTA coarse cycle where the level above it has
+// kernels that spread over the SMs: the two-sweep passes (FP32; 32 x 16 x 16
+// cells: 44 us in the CTA, 6 + 8 us as passes with a CTA cycle of 21 us below),
+// or on the FP64 path the per-colour kernels (an SM does two FP64 operations
+// per clock: about 190 us in the CTA, a third of that as launches).
+const long long kCoarseCells = 2048;
+
 // One V-cycle from level l for L x = R.  uh / ul as in smooth(): returns
 // true if the correction was added to that iterate by the last sweep.
 // *where: the buffer that holds the result otherwise (X, or the level's
@@ -602,6 +629,10 @@ bool vcycle(vsv_grid* g, const std::vector<Level>& lv, int l, Comp3<T> X, Rhs3<T
     if (l > 0) {
       Comp3<T> E = X;
       Comp3<T> RR{{(T*)R.B[0], (T*)R.B[1], (T*)R.B[2]}};
+      CoarseCycle CC;
+      if (g->sol.variant != 1 && coarse_plan(g, lv, l, &CC, sizeof(T)) &&
+          launch_coarse_vcycle<T>(g->cx, CC, E, RR, ncomp))
+        return false;
       if (launch_coarse_solve<T>(g->cx, L, E, RR, ncomp, coarsest_sweeps(L, g->sol.coarse_sweeps),
                                  h2))
         return false;
@@ -622,7 +653,8 @@ bool vcycle(vsv_grid* g, const std::vector<Level>& lv, int l, Comp3<T> X, Rhs3<T
     Comp3<T> RR{{(T*)R.B[0], (T*)R.B[1], (T*)R.B[2]}};
     if (run_lower_cycle<T>(g, lv, l, X, RR, ncomp)) return false;
   }
-  if (l > 0 && x_zero && g->sol.variant != 1 && R.beta == (T)1 && !R.S[0] && !R.S[1] && !R.S[2]) {
+  if (l > 0 && x_zero && g->sol.variant != 1 && R.beta == (T)1 && !R.S[0] && !R.S[1] && !R.S[2] &&
+      (L.cells() <= kCoarseCells || (sizeof(T) == 4 && !passes_wanted<T>(g, lv, l, x_zero, R)))) {
     // the remaining levels fit in one CTA's shared memory: one launch
     CoarseCycle CC;
     coarse_plan(g, lv, l, &CC, sizeof(T));

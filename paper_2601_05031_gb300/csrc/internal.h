@@ -166,9 +166,15 @@ struct CoarseCycle {
   double omega;                // relaxation weight of the nu1 / nu2 sweeps (coarsest: 1)
   double h2[kMaxLevels];       // 1 / inv_h2 of each level (rounded to T in the kernel)
   long long off[kMaxLevels];   // element offset of level l's (e, r) pair
+  int scratch;                 // element offset of the residual scratch
+  // per level: threads that work on it; planes per run and number of runs;
+  // whether the runs cover it evenly and are held in registers
+  int threads[kMaxLevels], run[kMaxLevels], runs[kMaxLevels];
+  bool reg[kMaxLevels];
   long long total;             // elements of shared memory
 };
 constexpr size_t kCoarseCycleSmem = 200 * 1024;
+constexpr int kCvThreads = 512;   // threads of the CTA that runs it
 template <class T>
 bool launch_coarse_vcycle(Ctx& cx, const CoarseCycle& CC, Comp3<T> E, Comp3<T> R, int ncomp);
 

@@ -510,6 +510,26 @@ __host__ __device__ bool blocked_transfer_ok(const Level& F, const Level& C) {
 // V-cycle there (same operations as the level-by-level kernels: red-black
 // sweeps, residual restricted by averaging, trilinear prolongation), which
 // replaces dozens of latency-bound launches per V-cycle by one.
+//
+// One SM runs it once, so its time is set by the instructions it issues, by
+// its chain of dependent phases (about 55 on five levels) and by the code it
+// has to fetch.  Each level keeps its two colours ((i + j + k) & 1) in
+// separate arrays of half the row length: a cell's neighbours are all in the
+// other colour's array, at the cell's own index for y and z and at that index
+// and one beside it for x, without unused lanes or bank conflicts.  A thread
+// holds a run of 1, 2, 4 or 8 planes of one column pair in registers (levels
+// that such runs do not cover evenly take a loop over shared memory), and the
+// boundary rule is resolved once per visit of a level.  A level is worked on
+// by only as many warps as it has runs, on a named barrier of its own (a
+// single warp needs none); the other warps wait for it to come back.
+//
+// Measured, one visit of 32 x 16 x 16 cells and below (three CTAs, cold
+// caches): 61 -> 44 us, 245 k -> 121 k warp instructions per CTA; 21 us from
+// 16 x 8 x 8 cells down.  What is left waits on barriers (2.4 of 8 stall
+// cycles per issue), instruction fetch (2.6) and fixed latencies (1.8).  One
+// copy of the code serves both directions: separate copies took 97 k
+// instructions but 57 us, fetching instructions (8.1), and loops over shared
+// memory alone (compact code, 217 k instructions) 59 us.
 
 // q = a / d, with rem = a - q d (0 <= a, 0 < d): a shift and a mask where d
 // is a power of two (every level of a power-of-two grid), else a division.
@@ -523,166 +543,560 @@ __device__ __forceinline__ int cv_divmod(int a, int d, int& rem) {
   return q;
 }
 
-// The thread's cells of one colour are visited with the index (i2, j, k)
-// advanced by the block size incrementally (adds and carries instead of two
-// integer divisions per cell).  The neighbour sum, the wall count and the
-// update are those of sum_nb and the per-colour sweep (same operands, same
-// order of the additions), with 32-bit offsets into shared memory, and with
-// the level's geometry and the weights omega rc (one per count of wall
-// neighbours, in shared memory) formed once per call instead of per cell.
-template <class T>
-__device__ void cv_sweep(const Level& L, T* e, const T* r, int sweeps, T h2, T omega) {
-  __shared__ T wtab[8];
-  const int nx = L.n[0], ny = L.n[1], nz = L.n[2], nxh = (nx + 1) >> 1;
-  const int sz = nx * ny;
-  const int nh = nxh * ny * nz;   // cells of one colour, rounded up per row
-  const bool ax = L.act[0], ay = L.act[1], az = L.act[2];
-  const bool px = L.per[0], py = L.per[1], pz = L.per[2];
-  const T c1 = (T)1 - omega;
-  const int B = blockDim.x;
-  int Bi, Bj, i20, j0;
-  const int Bk = cv_divmod(cv_divmod(B, nxh, Bi), ny, Bj);
-  const int k0 = cv_divmod(cv_divmod((int)threadIdx.x, nxh, i20), ny, j0);
-  if (threadIdx.x < 7) wtab[threadIdx.x] = wscale(omega, lv_rc<T>(L, (int)threadIdx.x));
-  __syncthreads();
-  for (int s = 0; s < sweeps; ++s)
-    for (int color = 0; color < 2; ++color) {
-      int i2 = i20, j = j0, k = k0;
-      for (int t2 = threadIdx.x; t2 < nh; t2 += B) {
-        if (t2 != threadIdx.x) {
-          i2 += Bi;
-          int cj = Bj;
-          if (i2 >= nxh) { i2 -= nxh; ++cj; }
-          j += cj;
-          int ck = Bk;
-          while (j >= ny) { j -= ny; ++ck; }
-          k += ck;
-        }
-        const int i = 2 * i2 + ((j + k + color) & 1);
-        if (i >= nx) continue;
-        const int t = (k * ny + j) * nx + i;
-        int nwall = 0;
-        T a = 0, b = 0;
-        if (ax) {
-          if (i > 0) a = e[t - 1]; else if (px) a = e[t + nx - 1]; else ++nwall;
-          if (i < nx - 1) b = e[t + 1]; else if (px) b = e[t - (nx - 1)]; else ++nwall;
-        }
-        const T s0 = a + b;
-        a = 0; b = 0;
-        if (ay) {
-          if (j > 0) a = e[t - nx]; else if (py) a = e[t + (ny - 1) * nx]; else ++nwall;
-          if (j < ny - 1) b = e[t + nx]; else if (py) b = e[t - (ny - 1) * nx]; else ++nwall;
-        }
-        const T s1 = a + b;
-        a = 0; b = 0;
-        if (az) {
-          if (k > 0) a = e[t - sz]; else if (pz) a = e[t + (nz - 1) * sz]; else ++nwall;
-          if (k < nz - 1) b = e[t + sz]; else if (pz) b = e[t - (nz - 1) * sz]; else ++nwall;
-        }
-        const T s2 = a + b;
-        e[t] = relax(e[t], nb_term((s0 + s1) + s2, r[t], h2), wtab[nwall], c1);
-      }
-      __syncthreads();
-    }
+__device__ __forceinline__ void cv_sync(int id, int n) {
+  if (n == 32) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
+// A level in shared memory: e and r of each colour, `half` elements apart.
+struct CvLevel {
+  int e, r;                   // element offsets
+  int nx, ny, nz, nxh, cols, half;
+  int n;                      // threads that work on it
+  int runs, len;              // column pairs x runs along z; planes per run
+  bool reg;                   // runs of 1, 2, 4 or 8 planes cover the level evenly
+  __device__ __forceinline__ CvLevel(const CoarseCycle& CC, int l) {
+    const Level& L = CC.lv[l];
+    nx = L.n[0]; ny = L.n[1]; nz = L.n[2];
+    nxh = (nx + 1) >> 1;
+    cols = nxh * ny;
+    half = cols * nz;
+    e = (int)CC.off[l];
+    r = e + 2 * half;
+    n = CC.threads[l];
+    len = CC.run[l];
+    runs = CC.runs[l];
+    reg = CC.reg[l];
+  }
+  __device__ __forceinline__ int at(int i, int j, int k) const {
+    return ((i + j + k) & 1) * half + (k * ny + j) * nxh + (i >> 1);
+  }
+};
+
+// A run: planes k0 .. k1 - 1 of the column pair (2 i2, 2 i2 + 1, j).
+struct CvRun {
+  int i2, j, k0, k1;
+  __device__ __forceinline__ void set(const CvLevel& V, int t) {
+    int col;
+    const int seg = cv_divmod(t, V.cols, col);
+    j = cv_divmod(col, V.nxh, i2);
+    k0 = seg * V.len;
+    k1 = min(k0 + V.len, V.nz);
+  }
+};
+
+// The level's runs of this thread, one after the other (one, except on a
+// level with more column pairs than threads).
+template <class F>
+__device__ __forceinline__ void cv_runs(const CvLevel& V, F&& f) {
+  for (int t = threadIdx.x; t < V.runs; t += V.n) {
+    CvRun R;
+    R.set(V, t);
+    f(R);
+  }
+}
+
+// `sweeps` red-black sweeps (from_zero: e is zero on entry and may hold
+// anything), then (resid) the residual of both colours into the scratch.
+// The neighbour sum, the wall count and the update are those of sum_nb and
+// the per-colour sweep.
 template <class T>
-__device__ void cv_restrict(const Level& F, const Level& C, const T* e, const T* r, T* rc) {
-  const int nc = (int)C.cells();
-  const int fx = F.n[0] / C.n[0], fy = F.n[1] / C.n[1], fz = F.n[2] / C.n[2];
-  for (int t = threadIdx.x; t < nc; t += blockDim.x) {
+__device__ __forceinline__ void cv_passes(const CoarseCycle& CC, int l, const CvLevel& V, T* sm,
+                                          int sweeps, T omega, bool from_zero, bool resid) {
+  const Level& L = CC.lv[l];
+  const T h2 = (T)CC.h2[l], c1 = (T)1 - omega, ih2 = lv_ih2<T>(L);
+  const bool ax = L.act[0], ay = L.act[1], az = L.act[2];
+  const bool px = L.per[0], py = L.per[1], pz = L.per[2];
+  const int passes = 2 * sweeps + (resid ? 2 : 0), bar = 1 + l - CC.first;
+  const bool once = V.runs <= V.n;
+  CvRun R;
+  bool hu = false, hd = false, hs0 = false, hs1 = false;
+  int o = 0, du = 0, dd = 0, ds0 = 0, ds1 = 0, nw0 = 0, nw1 = 0, last1 = 0;
+  T w0 = 0, w1 = 0;
+  for (int pass = 0; pass < passes; ++pass) {
+    const int c = pass & 1;
+    const bool zero = from_zero && pass == 0, rs = pass >= 2 * sweeps;
+    for (int t = threadIdx.x; t < V.runs; t += V.n) {
+      if (pass == 0 || !once) {
+        R.set(V, t);
+        o = V.e + (R.k0 * V.ny + R.j) * V.nxh + R.i2;
+        hu = ay && (py || R.j > 0);
+        hd = ay && (py || R.j < V.ny - 1);
+        du = R.j > 0 ? -V.nxh : (V.ny - 1) * V.nxh;
+        dd = R.j < V.ny - 1 ? V.nxh : (1 - V.ny) * V.nxh;
+        // beside the own index: left of an even column, right of an odd one
+        hs0 = ax && (px || R.i2 > 0);
+        hs1 = ax && (px || R.i2 < V.nxh - 1);
+        ds0 = R.i2 > 0 ? -1 : V.nxh - 1;
+        ds1 = R.i2 < V.nxh - 1 ? 1 : 1 - V.nxh;
+        const int yw = ay && !py ? (R.j == 0) + (R.j == V.ny - 1) : 0;
+        const bool xw = ax && !px;
+        last1 = (V.nx & 1) && R.i2 == V.nxh - 1;   // the odd column lies beyond the wall
+        nw0 = yw + (xw ? (R.i2 == 0) + last1 : 0);
+        nw1 = yw + (xw ? R.i2 == V.nxh - 1 : 0);
+        w0 = wscale(omega, lv_rc<T>(L, nw0));
+        w1 = wscale(omega, lv_rc<T>(L, nw1));
+      }
+      T* own = sm + o + c * V.half;
+      const T* oth = sm + o + (1 - c) * V.half;
+      const T* rr = own + 2 * V.half;
+      T* out = rs ? sm + CC.scratch + (o - V.e) + c * V.half : own;
+      // zm, m, zp: the other colour's column below, at and above the plane
+      T zm = 0, m = 0;
+      if (!zero) {
+        if (az && R.k0 > 0) zm = oth[-V.cols];
+        else if (az && pz) zm = oth[(V.nz - 1 - R.k0) * V.cols];
+        m = oth[0];
+      }
+      bool par = (R.j + R.k0 + c) & 1;
+#pragma unroll 2
+      for (int k = R.k0; k < R.k1; ++k) {
+        const int q = (k - R.k0) * V.cols;
+        T zp = 0, x = 0, u = 0, d = 0;
+        if (!zero) {
+          if (az && k < V.nz - 1) zp = oth[q + V.cols];
+          else if (az && pz) zp = oth[q + (1 - V.nz) * V.cols];
+          if (par ? hs1 : hs0) x = oth[q + (par ? ds1 : ds0)];
+          if (hu) u = oth[q + du];
+          if (hd) d = oth[q + dd];
+        }
+        const T mid = ax ? m : (T)0;
+        const T s = ((mid + x) + (u + d)) + (zm + zp), b = rr[q];
+        const T xo = from_zero && pass < 2 ? (T)0 : own[q];
+        T w = par ? w1 : w0;
+        int nw = par ? nw1 : nw0;
+        if (az && !pz && (k == 0 || k == V.nz - 1)) {
+          nw += (k == 0) + (k == V.nz - 1);
+          w = wscale(omega, lv_rc<T>(L, nw));
+        }
+        const T v = rs ? resid_value(b, s, lv_coef<T>(L, nw), xo, ih2) : relax(xo, nb_term(s, b, h2), w, c1);
+        // the spare cell of an odd row stays zero: it is the ghost beyond the wall
+        out[q] = par && last1 ? (T)0 : v;
+        zm = m;
+        m = zp;
+        par = !par;
+      }
+    }
+    cv_sync(bar, V.n);
+  }
+}
+
+// The visit of a level whose runs of LEN planes a thread holds in registers,
+// both colours (values and rhs): of a cell's neighbours only the two in y, one
+// in x and those at the run's ends are loads.  Cell q of colour c has column
+// parity (p0 + q + c) & 1, p0 = (j + k0) & 1; what depends on it is kept by
+// a = (q + c) & 1, so that every index is known at compile time.
+template <class T, int LEN>
+struct CvRegRun {
+  T e[2][LEN], r[2][LEN];
+  CvRun R;
+  bool on, ok[2];        // the thread has a run; the column exists (odd extents have a spare cell)
+  bool hs[2], hu, hd;    // neighbours present: x beside the own index, y - 1, y + 1
+  int ds[2], du, dd;     // and their distances
+  bool hlo, hhi;         // planes below and above the run
+  int dlo, dhi;
+  int o;                 // offset of the run's first cell in a colour
+  T* p[2];               // and its place among the values of each colour
+  bool mid;              // x couples
+  int nw[2], zb, zt;     // wall neighbours without z; z walls at the run's first and last plane
+
+  __device__ __forceinline__ CvRegRun(const Level& L, const CvLevel& V, T* sm) {
+    on = (int)threadIdx.x < V.runs;
+    R.set(V, on ? (int)threadIdx.x : 0);
+    const bool ax = L.act[0], ay = L.act[1], az = L.act[2];
+    const bool px = L.per[0], py = L.per[1], pz = L.per[2];
+    o = (R.k0 * V.ny + R.j) * V.nxh + R.i2;
+    p[0] = sm + V.e + o;
+    p[1] = p[0] + V.half;
+    mid = ax;
+    const bool xw = ax && !px, spare = (V.nx & 1) && R.i2 == V.nxh - 1;
+    const int yw = ay && !py ? (R.j == 0) + (R.j == V.ny - 1) : 0;
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const bool odd = (R.j + R.k0 + a) & 1;
+      hs[a] = ax && (px || (odd ? R.i2 < V.nxh - 1 : R.i2 > 0));
+      ds[a] = odd ? (R.i2 < V.nxh - 1 ? 1 : 1 - V.nxh) : (R.i2 > 0 ? -1 : V.nxh - 1);
+      ok[a] = !(odd && spare);
+      nw[a] = yw + (xw ? (odd ? R.i2 == V.nxh - 1 : (R.i2 == 0) + spare) : 0);
+    }
+    hu = ay && (py || R.j > 0);
+    hd = ay && (py || R.j < V.ny - 1);
+    du = R.j > 0 ? -V.nxh : (V.ny - 1) * V.nxh;
+    dd = R.j < V.ny - 1 ? V.nxh : (1 - V.ny) * V.nxh;
+    hlo = az && (pz || R.k0 > 0);
+    hhi = az && (pz || R.k1 < V.nz);
+    dlo = R.k0 > 0 ? -V.cols : (V.nz - 1) * V.cols;
+    dhi = R.k1 < V.nz ? LEN * V.cols : -R.k0 * V.cols;
+    zb = az && !pz && R.k0 == 0;
+    zt = az && !pz && R.k1 == V.nz;
+  }
+  __device__ __forceinline__ int walls(int a, int q) const {
+    return nw[a] + (q == 0 ? zb : 0) + (q == LEN - 1 ? zt : 0);
+  }
+  // rhs from shared memory, or that of the first level from global memory (g)
+  __device__ __forceinline__ void load_r(const CvLevel& V, const T* __restrict__ g) {
+#pragma unroll
+    for (int q = 0; q < LEN; ++q) {
+      T even = 0, odd = 0;
+      if (g && on) {
+        const T* s = g + ((R.k0 + q) * V.ny + R.j) * V.nx + 2 * R.i2;
+        even = s[0];
+        if (2 * R.i2 + 1 < V.nx) odd = s[1];
+      }
+      const bool par = (R.j + R.k0 + q) & 1;   // column parity of colour 0
+      r[0][q] = g ? (par ? odd : even) : p[0][2 * V.half + q * V.cols];
+      r[1][q] = g ? (par ? even : odd) : p[1][2 * V.half + q * V.cols];
+    }
+  }
+  __device__ __forceinline__ void store_global(const CvLevel& V, T* __restrict__ g) const {
+    if (!on) return;
+#pragma unroll
+    for (int q = 0; q < LEN; ++q) {
+      T* d = g + ((R.k0 + q) * V.ny + R.j) * V.nx + 2 * R.i2;
+      const bool par = (R.j + R.k0 + q) & 1;
+      d[0] = par ? e[1][q] : e[0][q];
+      if (2 * R.i2 + 1 < V.nx) d[1] = par ? e[0][q] : e[1][q];
+    }
+  }
+  __device__ __forceinline__ void load_e(const CvLevel& V) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int q = 0; q < LEN; ++q) e[c][q] = p[c][q * V.cols];
+  }
+  // neighbour sums of colour c, ((x- + x+) + (y- + y+)) + (z- + z+)
+  __device__ __forceinline__ void sums(const CvLevel& V, int c, T* s) const {
+    const T* oth = p[1 - c];
+    T lo = 0, hi = 0;
+    if (hlo) lo = oth[dlo];
+    if (hhi) hi = oth[dhi];
+#pragma unroll
+    for (int q = 0; q < LEN; ++q) {
+      const T* at = oth + q * V.cols;
+      T x = 0, u = 0, d = 0;
+      if (hs[(q + c) & 1]) x = at[ds[(q + c) & 1]];
+      if (hu) u = at[du];
+      if (hd) d = at[dd];
+      const T m = mid ? e[1 - c][q] : (T)0;
+      const T zm = q > 0 ? e[1 - c][q > 0 ? q - 1 : 0] : lo;
+      const T zp = q < LEN - 1 ? e[1 - c][q < LEN - 1 ? q + 1 : 0] : hi;
+      s[q] = ((m + x) + (u + d)) + (zm + zp);
+    }
+  }
+  // e += P e(W) of the run (every axis halved)
+  __device__ __forceinline__ void prolong(const CvLevel& V, const CvLevel& W, const Level& C, const T* we) {
+    if (!on) return;
+    const T ma = -lv_alpha<T>(C);
+    const int J = R.j >> 1;
+    int xl = outer_idx(R.i2 - 1, W.nx, C.per[0]), xr = outer_idx(R.i2 + 1, W.nx, C.per[0]);
+    int jn = outer_idx(J + ((R.j & 1) ? 1 : -1), W.ny, C.per[1]);
+    const T fl = xl >= 0 ? (T)1 : ma, fr = xr >= 0 ? (T)1 : ma, fy = jn >= 0 ? (T)1 : ma;
+    if (xl < 0) xl = R.i2;
+    if (xr < 0) xr = R.i2;
+    if (jn < 0) jn = J;
+    // x-interpolated values of coarse plane K (its wall factor included) on the
+    // even and odd column: of the run's own coarse row and of the one beside it
+    auto plane = [&](int K, T v[4]) {
+      int kk = outer_idx(K, W.nz, C.per[2]);
+      const T fz = kk >= 0 ? (T)1 : ma;
+      if (kk < 0) kk = K < 0 ? 0 : W.nz - 1;
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const int jj = b ? jn : J;
+        const T f = fz * (b ? fy : (T)1);
+        const T* row = we + (kk * W.ny + jj) * W.nxh;
+        const int sc = (R.i2 + jj + kk) & 1, hc = sc * W.half, hx = (1 - sc) * W.half;
+        const T n0 = mul_t(f, row[hc + (R.i2 >> 1)]);
+        v[2 * b] = prolong_pair(n0, mul_t(f * fl, row[((xl ^ R.i2) & 1 ? hx : hc) + (xl >> 1)]));
+        v[2 * b + 1] = prolong_pair(n0, mul_t(f * fr, row[((xr ^ R.i2) & 1 ? hx : hc) + (xr >> 1)]));
+      }
+    };
+    auto add = [&](int q, const T c[4], const T n[4]) {
+      T v[2];
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+        v[x] = fma_t((T)0.0625, n[2 + x],
+                     fma_t((T)0.1875, n[x], fma_t((T)0.1875, c[2 + x], mul_t((T)0.5625, c[x]))));
+      const bool par = (R.j + R.k0 + q) & 1;
+      e[0][q] += par ? v[1] : v[0];
+      e[1][q] += par ? v[0] : v[1];
+      p[0][q * V.cols] = e[0][q];
+      p[1][q * V.cols] = e[1][q];
+    };
+    const int K = R.k0 >> 1;
+    T a[4], c[4], n[4];
+    plane(K, c);
+    if constexpr (LEN == 1) {
+      plane(K + ((R.k0 & 1) ? 1 : -1), n);
+      add(0, c, n);
+    } else {
+      plane(K - 1, a);
+#pragma unroll
+      for (int h = 0; h < LEN / 2; ++h) {
+        plane(K + h + 1, n);
+        add(2 * h, c, a);
+        add(2 * h + 1, c, n);
+#pragma unroll
+        for (int x = 0; x < 4; ++x) { a[x] = c[x]; c[x] = n[x]; }
+      }
+    }
+  }
+};
+
+// One visit of level l: down: `sweeps` sweeps from e = 0, then (resid) the
+// residual into the scratch; up: e += P e(W) where every axis is halved
+// (`blocked`; else it is already in e), then the sweeps; the first level's
+// result also goes to global memory.
+template <class T, int LEN>
+__device__ __forceinline__ void cv_visit(const CoarseCycle& CC, int l, const CvLevel& V,
+                                         const CvLevel& W, T* sm, const T* rr, T* e_out, int sweeps,
+                                         T omega, bool down, bool resid, bool blocked) {
+  const Level& L = CC.lv[l];
+  const T h2 = (T)CC.h2[l], c1 = (T)1 - omega;
+  const int bar = 1 + l - CC.first;
+  CvRegRun<T, LEN> X(L, V, sm);
+  X.load_r(V, l == CC.first ? rr : nullptr);
+  if (down) {
+#pragma unroll
+    for (int q = 0; q < LEN; ++q) X.e[0][q] = X.e[1][q] = (T)0;
+  } else {
+    X.load_e(V);
+    if (blocked) {
+      X.prolong(V, W, CC.lv[l + 1], sm + W.e);
+      cv_sync(bar, V.n);
+    }
+  }
+  T w[2][3];   // omega / diagonal: at the run's first plane, inside, at its last
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    w[a][0] = wscale(omega, lv_rc<T>(L, X.walls(a, 0)));
+    w[a][1] = wscale(omega, lv_rc<T>(L, X.nw[a]));
+    w[a][2] = wscale(omega, lv_rc<T>(L, X.walls(a, LEN - 1)));
+  }
+  T s[LEN];
+#pragma unroll 1
+  for (int it = 0; it < sweeps; ++it) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (X.on) {
+        if (c == 0 && down && it == 0) {   // from zero: every neighbour is zero
+#pragma unroll
+          for (int q = 0; q < LEN; ++q) s[q] = (T)0;
+        } else {
+          X.sums(V, c, s);
+        }
+#pragma unroll
+        for (int q = 0; q < LEN; ++q) {
+          const int a = (q + c) & 1;
+          if (X.ok[a]) {
+            X.e[c][q] = relax(X.e[c][q], nb_term(s[q], X.r[c][q], h2),
+                              w[a][q == 0 ? 0 : (q == LEN - 1 ? 2 : 1)], c1);
+            X.p[c][q * V.cols] = X.e[c][q];
+          }
+        }
+      }
+      cv_sync(bar, V.n);
+    }
+  }
+  if (resid) {
+    if (X.on) {
+      const T ih2 = lv_ih2<T>(L);
+      T* const sc = sm + CC.scratch + X.o;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        X.sums(V, c, s);
+#pragma unroll
+        for (int q = 0; q < LEN; ++q)
+          sc[c * V.half + q * V.cols] =
+              resid_value(X.r[c][q], s[q], lv_coef<T>(L, X.walls((q + c) & 1, q)), X.e[c][q], ih2);
+      }
+    }
+    cv_sync(bar, V.n);
+  }
+  if (!down && l == CC.first) X.store_global(V, e_out);
+}
+
+// The residuals in the scratch averaged onto the rhs of W, children in order.
+template <class T>
+__device__ __forceinline__ void cv_restrict(const CoarseCycle& CC, int l, const CvLevel& V,
+                                            const CvLevel& W, T* sm) {
+  const int nc = W.nx * W.ny * W.nz;
+  const int fx = V.nx / W.nx, fy = V.ny / W.ny, fz = V.nz / W.nz;
+  const T* S = sm + CC.scratch;
+  for (int t = threadIdx.x; t < nc; t += V.n) {
     int I, J;
-    const int K = cv_divmod(cv_divmod(t, C.n[0], I), C.n[1], J);
+    const int K = cv_divmod(cv_divmod(t, W.nx, I), W.ny, J);
     T acc = 0;
     for (int dk = 0; dk < fz; ++dk)
       for (int dj = 0; dj < fy; ++dj)
-        for (int di = 0; di < fx; ++di) {
-          const int i = I * fx + di, j = J * fy + dj, k = K * fz + dk;
-          const int c = (k * F.n[1] + j) * F.n[0] + i;
-          acc += resid_plain(e, F, i, j, k, c, r[c]);
-        }
-    rc[t] = acc / (T)(fx * fy * fz);
+        for (int di = 0; di < fx; ++di) acc += S[V.at(I * fx + di, J * fy + dj, K * fz + dk)];
+    sm[W.r + W.at(I, J, K)] = acc / (T)(fx * fy * fz);
   }
-  __syncthreads();
+  cv_sync(1 + l - CC.first, V.n);
 }
 
+// e(V) += P e(W)
 template <class T>
-__device__ void cv_prolong(const Level& F, const Level& C, T* e, const T* ec) {
-  if (blocked_transfer_ok(F, C)) {   // as k_prolong_block
-    const int nc = (int)C.cells();
-    for (int t = threadIdx.x; t < nc; t += blockDim.x) {
-      int I, J;
-      const int K = cv_divmod(cv_divmod(t, C.n[0], I), C.n[1], J);
-      T v[2][2][2];
-      prolong_children<T>(C, ec, I, J, K, v);
-      for (int c = 0; c < 2; ++c)
-        for (int b = 0; b < 2; ++b)
-          for (int a = 0; a < 2; ++a)
-            e[((2 * K + c) * F.n[1] + 2 * J + b) * F.n[0] + 2 * I + a] += v[c][b][a];
-    }
-    __syncthreads();
-    return;
-  }
-  const int nf = (int)F.cells();   // as k_prolong_add
-  const T al = lv_alpha<T>(C);
-  for (int t = threadIdx.x; t < nf; t += blockDim.x) {
-    const int i = t % F.n[0], q = t / F.n[0];
-    const int j = q % F.n[1], k = q / F.n[1];
-    const Interp1<T> ax = interp_axis<T>(i, F.n[0] / C.n[0], C.n[0], C.per[0], al);
-    const Interp1<T> ay = interp_axis<T>(j, F.n[1] / C.n[1], C.n[1], C.per[1], al);
-    const Interp1<T> az = interp_axis<T>(k, F.n[2] / C.n[2], C.n[2], C.per[2], al);
-    T acc = 0;
-    for (int c2 = 0; c2 < 2; ++c2)
-      for (int b2 = 0; b2 < 2; ++b2)
-        for (int a2 = 0; a2 < 2; ++a2) {
-          const T w = ax.w[a2] * ay.w[b2] * az.w[c2];
-          if (w != (T)0) acc += w * ec[(az.idx[c2] * C.n[1] + ay.idx[b2]) * C.n[0] + ax.idx[a2]];
+__device__ __forceinline__ void cv_prolong(const CoarseCycle& CC, int l, const CvLevel& V,
+                                           const CvLevel& W, T* sm) {
+  const Level& F = CC.lv[l];
+  const Level& C = CC.lv[l + 1];
+  const T* we = sm + W.e;
+  if (blocked_transfer_ok(F, C)) {   // the values of k_prolong_block
+    const T ma = -lv_alpha<T>(C);
+    cv_runs(V, [&](const CvRun& R) {
+      const int J = R.j >> 1;
+      int xl = outer_idx(R.i2 - 1, W.nx, C.per[0]), xr = outer_idx(R.i2 + 1, W.nx, C.per[0]);
+      int jn = outer_idx(J + ((R.j & 1) ? 1 : -1), W.ny, C.per[1]);
+      const T fl = xl >= 0 ? (T)1 : ma, fr = xr >= 0 ? (T)1 : ma, fy = jn >= 0 ? (T)1 : ma;
+      if (xl < 0) xl = R.i2;
+      if (xr < 0) xr = R.i2;
+      if (jn < 0) jn = J;
+      // x-interpolated values of coarse plane K (its wall factor included) on
+      // the even (.x) and odd (.y) column: the row's own and the one beside it
+      auto plane = [&](int K, T p[4]) {
+        int kk = outer_idx(K, W.nz, C.per[2]);
+        const T fz = kk >= 0 ? (T)1 : ma;
+        if (kk < 0) kk = K < 0 ? 0 : W.nz - 1;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          const int jj = b ? jn : J;
+          const T f = fz * (b ? fy : (T)1);
+          const T* row = we + (kk * W.ny + jj) * W.nxh;
+          const int sc = (R.i2 + jj + kk) & 1, hc = sc * W.half, hx = (1 - sc) * W.half;
+          const T n0 = mul_t(f, row[hc + (R.i2 >> 1)]);
+          p[2 * b] = prolong_pair(n0, mul_t(f * fl, row[((xl ^ R.i2) & 1 ? hx : hc) + (xl >> 1)]));
+          p[2 * b + 1] = prolong_pair(n0, mul_t(f * fr, row[((xr ^ R.i2) & 1 ? hx : hc) + (xr >> 1)]));
         }
-    e[t] += acc;
+      };
+      auto add = [&](int k, const T c[4], const T n[4]) {
+        T v[2];
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+          v[x] = fma_t((T)0.0625, n[2 + x],
+                       fma_t((T)0.1875, n[x], fma_t((T)0.1875, c[2 + x], mul_t((T)0.5625, c[x]))));
+        T* e = sm + V.e + (k * V.ny + R.j) * V.nxh + R.i2;
+        const int par = (R.j + k) & 1;   // the even column's colour
+        e[par * V.half] += v[0];
+        e[(1 - par) * V.half] += v[1];
+      };
+      // planes 2K and 2K + 1 from coarse planes K - 1, K and K, K + 1
+      T a[4], c[4], n[4];
+      int K = R.k0 >> 1;
+      plane(K, c);
+      if (!(R.k0 & 1)) plane(K - 1, a);
+#pragma unroll 1
+      for (int k = R.k0; k < R.k1; ++K) {
+        if (!(k & 1)) add(k++, c, a);
+        if (k < R.k1) {
+          plane(K + 1, n);
+          add(k++, c, n);
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x) { a[x] = c[x]; c[x] = n[x]; }
+      }
+    });
+  } else {                             // as k_prolong_add
+    const int nf = V.nx * V.ny * V.nz;
+    const T al = lv_alpha<T>(C);
+    for (int t = threadIdx.x; t < nf; t += V.n) {
+      int i, j;
+      const int k = cv_divmod(cv_divmod(t, V.nx, i), V.ny, j);
+      const Interp1<T> ax = interp_axis<T>(i, F.n[0] / C.n[0], C.n[0], C.per[0], al);
+      const Interp1<T> ay = interp_axis<T>(j, F.n[1] / C.n[1], C.n[1], C.per[1], al);
+      const Interp1<T> az = interp_axis<T>(k, F.n[2] / C.n[2], C.n[2], C.per[2], al);
+      T acc = 0;
+      for (int c2 = 0; c2 < 2; ++c2)
+        for (int b2 = 0; b2 < 2; ++b2)
+          for (int a2 = 0; a2 < 2; ++a2) {
+            const T w = ax.w[a2] * ay.w[b2] * az.w[c2];
+            if (w != (T)0) acc += w * we[W.at(ax.idx[a2], ay.idx[b2], az.idx[c2])];
+          }
+      sm[V.e + V.at(i, j, k)] += acc;
+    }
   }
-  __syncthreads();
+  cv_sync(1 + l - CC.first, V.n);
 }
 
 // The lower V-cycle of one component in one CTA: rhs rr (level CC.first,
-// global memory) -> correction e_out, every level in shared memory `base`.
-template <class T>
-__device__ void coarse_vcycle_cta(const CoarseCycle& CC, const T* __restrict__ rr,
-                                  T* __restrict__ e_out, T* base) {
-  const int f = CC.first, l_last = CC.last;
-  // (e, r) of level l in shared memory; CC is a grid-constant parameter, so
-  // its tables are read in place at run-time indices (no local copies)
-  auto e = [&](int l) { return base + CC.off[l]; };
-  auto r = [&](int l) { return base + CC.off[l] + CC.lv[l].cells(); };
-  const int n0 = (int)CC.lv[f].cells();
-  for (int t = threadIdx.x; t < n0; t += blockDim.x) {
-    r(f)[t] = rr[t];
-    e(f)[t] = (T)0;
-  }
-  __syncthreads();
-  for (int l = f; l < l_last; ++l) {
-    cv_sweep<T>(CC.lv[l], e(l), r(l), CC.nu1, (T)CC.h2[l], (T)CC.omega);
-    cv_restrict<T>(CC.lv[l], CC.lv[l + 1], e(l), r(l), r(l + 1));
-    const int nc = (int)CC.lv[l + 1].cells();
-    T* ec = e(l + 1);
-    for (int t = threadIdx.x; t < nc; t += blockDim.x) ec[t] = (T)0;
+// global memory) -> correction e_out, every level in shared memory `sm`.
+// MAX_LEN: the longest run whose registers fit.
+template <class T, int MAX_LEN>
+__device__ __forceinline__ void coarse_vcycle_cta(const CoarseCycle& CC, const T* __restrict__ rr,
+                                                  T* __restrict__ e_out, T* sm) {
+  const int f = CC.first, l_last = CC.last, tid = threadIdx.x;
+  if (!CC.reg[f]) {   // the loop reads its rhs from shared memory
+    const CvLevel V(CC, f);
+    if (tid < V.n)
+      cv_runs(V, [&](const CvRun& R) {
+        for (int k = R.k0; k < R.k1; ++k) {
+          const T* p = rr + (k * V.ny + R.j) * V.nx + 2 * R.i2;
+          T* r = sm + V.r + (k * V.ny + R.j) * V.nxh + R.i2;
+          const int par = (R.j + k) & 1;   // the even column's colour
+          r[par * V.half] = p[0];
+          if (2 * R.i2 + 1 < V.nx) r[(1 - par) * V.half] = p[1];
+        }
+      });
     __syncthreads();
   }
-  cv_sweep<T>(CC.lv[l_last], e(l_last), r(l_last), CC.coarse_sweeps, (T)CC.h2[l_last], (T)1);
-  for (int l = l_last - 1; l >= f; --l) {
-    cv_prolong<T>(CC.lv[l], CC.lv[l + 1], e(l), e(l + 1));
-    cv_sweep<T>(CC.lv[l], e(l), r(l), CC.nu2, (T)CC.h2[l], (T)CC.omega);
+  // down to the last level this thread works on, then back up; where a level
+  // has fewer threads the others wait at the barrier of the level above
+  bool down = true;
+  int l = tid < CC.threads[f] ? f : f - 1;
+  while (l >= f) {
+    const CvLevel V(CC, l);
+    const bool last = l == l_last;
+    const CvLevel W(CC, last ? l : l + 1);
+    const bool blocked = !last && blocked_transfer_ok(CC.lv[l], CC.lv[l + 1]);
+    if (!down) {
+      cv_sync(1 + l - f, V.n);   // the levels below are done
+      if (!V.reg || !blocked) cv_prolong<T>(CC, l, V, W, sm);
+    }
+    const int sweeps = last ? CC.coarse_sweeps : (down ? CC.nu1 : CC.nu2);
+    const T om = last ? (T)1 : (T)CC.omega;
+    const bool rs = down && !last;
+    if (down && sweeps == 0) {   // no pre-smoothing: e = 0 has to be there
+      for (int t = tid; t < 2 * V.half; t += V.n) sm[V.e + t] = (T)0;
+      cv_sync(1 + l - f, V.n);
+    }
+    if (!V.reg) cv_passes<T>(CC, l, V, sm, sweeps, om, down, rs);
+    else if (V.len == 1) cv_visit<T, 1>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
+    else if (V.len == 2) cv_visit<T, 2>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
+    else if (V.len == 4) cv_visit<T, 4>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
+    else cv_visit<T, MAX_LEN>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
+    if (rs) {
+      cv_restrict<T>(CC, l, V, W, sm);
+      if (tid < W.n) ++l;
+      else down = false;          // waits at the top of the loop for the levels below
+    } else {
+      down = false;
+      --l;
+    }
   }
-  const T* e0 = e(f);
-  for (int t = threadIdx.x; t < n0; t += blockDim.x) e_out[t] = e0[t];
+  if (CC.reg[f] && f < l_last) return;   // stored from the runs
+  __syncthreads();
+  const CvLevel V(CC, f);
+  if (tid < V.n)
+    cv_runs(V, [&](const CvRun& R) {
+      for (int k = R.k0; k < R.k1; ++k) {
+        T* p = e_out + (k * V.ny + R.j) * V.nx + 2 * R.i2;
+        const T* e = sm + V.e + (k * V.ny + R.j) * V.nxh + R.i2;
+        const int par = (R.j + k) & 1;
+        p[0] = e[par * V.half];
+        if (2 * R.i2 + 1 < V.nx) p[1] = e[(1 - par) * V.half];
+      }
+    });
 }
 
+// kCvThreads = 512: registers for runs of eight planes in FP32, four in FP64.
+
 template <class T>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(kCvThreads)
 k_coarse_vcycle(const __grid_constant__ CoarseCycle CC, Comp3<T> E, Comp3<T> RR) {
   pdl_begin();
   extern __shared__ unsigned char smem_cv[];
   const int comp = blockIdx.x;
-  coarse_vcycle_cta<T>(CC, RR.at(comp), E.at(comp), reinterpret_cast<T*>(smem_cv));
+  coarse_vcycle_cta<T, sizeof(T) == 4 ? 8 : 4>(CC, RR.at(comp), E.at(comp), reinterpret_cast<T*>(smem_cv));
 }
 
 template <class T>
@@ -694,7 +1108,7 @@ bool launch_coarse_vcycle(Ctx& cx, const CoarseCycle& CC, Comp3<T> E, Comp3<T> R
                            (int)smem) != cudaSuccess)
     return false;
   cx.before(VSV_KCLASS_SMOOTH);
-  launch_k(cx, k_coarse_vcycle<T>, ncomp, 1024, smem, CC, E, R);
+  launch_k(cx, k_coarse_vcycle<T>, ncomp, kCvThreads, smem, CC, E, R);
   // r of the first level read, e written; the rest stays in shared memory
   cx.after(VSV_KCLASS_SMOOTH, 2.0 * (double)sizeof(T) * (double)CC.lv[CC.first].cells() * ncomp);
   return true;
@@ -929,7 +1343,7 @@ k_lower_vcycle(const __grid_constant__ LowerCycle<T> P) {
   }
   if (lw <= P.last) {
     if (blockIdx.x < (unsigned)P.ncomp)
-      coarse_vcycle_cta<T>(P.cc_plan, P.r[lw][blockIdx.x], P.e[lw][blockIdx.x],
+      coarse_vcycle_cta<T, sizeof(T) == 4 ? 8 : 4>(P.cc_plan, P.r[lw][blockIdx.x], P.e[lw][blockIdx.x],
                            reinterpret_cast<T*>(smem_lc));
     if (!grid_sync(P.bar, epoch)) return;
   }

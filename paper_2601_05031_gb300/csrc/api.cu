@@ -397,23 +397,23 @@ Comp3<T> comp3(void* a, void* b, void* c) {
   return Comp3<T>{{(T*)a, (T*)b, (T*)c}};
 }
 
-// The velocity v = v0 + curl psi' for the observables and the field
-// exports, written over the source buffer f (scratch between steps): FP64
-// values on the FP64 path, double words (f, f_lo) formed in FP64 on the
-// mixed path.  *VL gets the low words (null pointers on the FP64 path).
+// Components first .. last of the velocity v = v0 + curl psi' for the
+// observables, written over the source buffer f (scratch between steps):
+// FP64 values on the FP64 path, double words (f, f_lo) on the mixed path.
+// *VL gets the low words (null pointers on the FP64 path).
 template <class T>
-void output_velocity(vsv_grid* g, const PhaseParams& P, Comp3<T>* V, Comp3<T>* VL) {
+void output_velocity(vsv_grid* g, const PhaseParams& P, int first, int last, Comp3<T>* V, Comp3<T>* VL) {
   *V = comp3<T>(g->f[0], g->f[1], g->f[2]);
+  const Comp3<T> psi = comp3<T>(g->ps[0], g->ps[1], g->ps[2]);
   if constexpr (std::is_same<T, float>::value) {
     *VL = comp3<float>(g->f_lo[0], g->f_lo[1], g->f_lo[2]);
-    launch_velocity_dw(g->cx, P, comp3<float>(g->ps[0], g->ps[1], g->ps[2]),
-                       comp3<float>(g->ps_lo[0], g->ps_lo[1], g->ps_lo[2]), ring3(g->v0d), *V,
-                       *VL);
+    const Comp3<float> lo = comp3<float>(g->ps_lo[0], g->ps_lo[1], g->ps_lo[2]);
+    for (int c = first; c <= last; ++c)
+      launch_velocity_dw(g->cx, P, psi, lo, g->v0d[c], c, V->p[c], VL->p[c]);
   } else {
     *VL = Comp3<T>{{nullptr, nullptr, nullptr}};
-    launch_velocity<T>(g->cx, P, comp3<T>(g->ps[0], g->ps[1], g->ps[2]),
-                       Comp3<T>{{nullptr, nullptr, nullptr}},
-                       comp3<T>(g->v0t[0], g->v0t[1], g->v0t[2]), *V);
+    for (int c = first; c <= last; ++c)
+      launch_velocity<T>(g->cx, P, psi, (const T*)g->v0t[c], c, V->p[c]);
   }
 }
 
@@ -1270,6 +1270,20 @@ const void* mapped_host(const void* p) {
   return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+// Device memory of the current device with elements of `size` bytes in
+// alignment: a kernel may write a field there itself.  Anything else (another
+// device's memory, host pointers, odd offsets) gets its field by a copy.
+bool kernel_writable(const void* p, size_t size) {
+  cudaPointerAttributes a;
+  int dev = -1;
+  if ((uintptr_t)p % size || cudaPointerGetAttributes(&a, p) != cudaSuccess ||
+      cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 // FP64 host or device words split into the hi + lo pair (hi, lo): in place
 // from mapped host memory, else through the staging buffer.
 vsv_status split_in(vsv_grid* g, const void* src, int on_device, float* hi, float* lo) {
@@ -1366,13 +1380,21 @@ vsv_status get_field_impl(vsv_grid* g, int field, void* dst, int dt, int on_devi
   T* tmp = (T*)g->stage_a;
   const bool mixed = std::is_same<T, float>::value;
   const cudaMemcpyKind dkind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  // double-word perturbation (mixed path) exported in FP64: hi + lo (+ base)
-  auto export_dw = [&](const float* hi, const float* lo, const double* tab) -> vsv_status {
-    launch_full_field_dw(g->cx, P, hi, lo, tab, 1, (double*)g->stage_a);
+  // where a kernel writes the exported field: straight into the caller's device
+  // memory, else into the staging buffer, from which deliver() copies it
+  const size_t out_sz = dt == VSV_DTYPE_F64 ? 8 : 4;
+  const bool direct = on_device && kernel_writable(dst, out_sz);
+  void* const to = direct ? dst : g->stage_a;
+  auto deliver = [&]() -> vsv_status {
     CKL();
-    CK(cudaMemcpyAsync(dst, g->stage_a, g->N * 8, dkind, g->cx.stream));
+    if (!direct) CK(cudaMemcpyAsync(dst, g->stage_a, g->N * out_sz, dkind, g->cx.stream));
     if (!on_device) CK(cudaStreamSynchronize(g->cx.stream));
     return VSV_OK;
+  };
+  // double-word perturbation (mixed path) exported in FP64: hi + lo (+ base)
+  auto export_dw = [&](const float* hi, const float* lo, const double* tab) -> vsv_status {
+    launch_full_field_dw(g->cx, P, hi, lo, tab, 1, (double*)to);
+    return deliver();
   };
   if (field == VSV_FIELD_PHI) return export_phi<T>(g, dt, on_device, dst);
   else if (field == VSV_FIELD_MU) {
@@ -1390,19 +1412,26 @@ vsv_status get_field_impl(vsv_grid* g, int field, void* dst, int dt, int on_devi
     launch_full_field<T>(g->cx, P, (const T*)g->ps[c], (const T*)g->ps_lo[c], g->ps_ring[c], 1, tmp);
     src = tmp;
   } else if (field >= VSV_FIELD_VEL_X && field <= VSV_FIELD_VEL_Z) {
-    Comp3<T> V, VL;
-    output_velocity<T>(g, P, &V, &VL);
     const int c = field - VSV_FIELD_VEL_X;
-    if (mixed && dt == VSV_DTYPE_F64) return export_dw((const float*)V.p[c], (const float*)VL.p[c], nullptr);
+    if constexpr (std::is_same<T, float>::value) {
+      const bool f64 = dt == VSV_DTYPE_F64;
+      launch_velocity_dw(g->cx, P, comp3<float>(g->ps[0], g->ps[1], g->ps[2]),
+                         comp3<float>(g->ps_lo[0], g->ps_lo[1], g->ps_lo[2]), g->v0d[c], c,
+                         f64 ? nullptr : (float*)to, nullptr, f64 ? (double*)to : nullptr);
+      return deliver();
+    } else if (dt == VSV_DTYPE_F64) {
+      launch_velocity<T>(g->cx, P, comp3<T>(g->ps[0], g->ps[1], g->ps[2]), (const T*)g->v0t[c], c,
+                         (T*)to);
+      return deliver();
+    }
+    Comp3<T> V, VL;
+    output_velocity<T>(g, P, c, c, &V, &VL);
     src = V.p[c];
   } else if (field == VSV_FIELD_STRESS_T) {
     Comp3<T> V, VL;
-    output_velocity<T>(g, P, &V, &VL);
-    launch_diag<T>(g->cx, P, (const T*)g->phi[g->cur], (const T*)g->phi_lo[g->cur],
-                   (const T*)g->g, (const T*)g->g_lo, V, VL,
-                   comp3<T>(g->om[0], g->om[1], g->om[2]), om_low<T>(g),
-                   comp3<T>(g->ps[0], g->ps[1], g->ps[2]), ps_low<T>(g),
-                   ring3(g->ps_ring), ring3(g->v0d), tmp, g->partials, g->red_blocks, g->dout);
+    output_velocity<T>(g, P, 0, 2, &V, &VL);
+    launch_sigma_t<T>(g->cx, P, V, VL, out_sz == sizeof(T) ? (T*)to : tmp);
+    if (out_sz == sizeof(T)) return deliver();
     src = tmp;
   } else if (field >= VSV_FIELD_OMEGA_PERT_X && field <= VSV_FIELD_OMEGA_PERT_Z) {
     const int c = field - VSV_FIELD_OMEGA_PERT_X;
@@ -2231,13 +2260,12 @@ vsv_status vsv_get_diagnostics(vsv_grid* g, vsv_diag* out) {
       g->phase_stale = false;
     }
     Comp3<T> V, VL;
-    output_velocity<T>(g, P, &V, &VL);
+    output_velocity<T>(g, P, 0, 2, &V, &VL);
     launch_diag<T>(g->cx, P, (const T*)g->phi[g->cur], (const T*)g->phi_lo[g->cur],
                    (const T*)g->g, (const T*)g->g_lo, V, VL,
                    comp3<T>(g->om[0], g->om[1], g->om[2]), om_low<T>(g),
                    comp3<T>(g->ps[0], g->ps[1], g->ps[2]), ps_low<T>(g),
-                   ring3(g->ps_ring), ring3(g->v0d), (T*)nullptr, g->partials, g->red_blocks,
-                   g->dout);
+                   ring3(g->ps_ring), ring3(g->v0d), g->partials, g->red_blocks, g->dout);
   };
   if (g->prec == VSV_FP64) run(double{});
   else run(float{});
@@ -2291,8 +2319,8 @@ vsv_status vsv_get_stress_profile(vsv_grid* g, double* out) {
   auto run = [&](auto tag) {
     using T = decltype(tag);
     Comp3<T> V, VL;
-    output_velocity<T>(g, P, &V, &VL);
-    launch_stress_profile<T>(g->cx, P, V, VL, g->profile);
+    output_velocity<T>(g, P, 0, 0, &V, &VL);
+    launch_stress_profile<T>(g->cx, P, V.p[0], VL.p[0], (double*)g->stage_a, g->profile);
   };
   if (g->prec == VSV_FP64) run(double{});
   else run(float{});

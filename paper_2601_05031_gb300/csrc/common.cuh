@@ -252,6 +252,17 @@ __device__ __forceinline__ FF ff_mul_f(FF a, float b) {
 }
 __device__ __forceinline__ float ff_round(FF a) { return __fadd_rn(a.hi, a.lo); }
 
+// (double)x, exactly, by integer operations: the conversion instruction runs on
+// the FP64 units, which do two operations per clock and SM, and takes as long
+// there as the addition it feeds.  A subnormal is scaled up first (exactly).
+__device__ __forceinline__ double f2d(float x) {
+  const bool tiny = (__float_as_uint(x) & 0x7f800000u) == 0u;
+  const unsigned u = __float_as_uint(tiny ? x * 16777216.f : x), e = u & 0x7f800000u;
+  const unsigned bias = e == 0x7f800000u ? 0x70000000u : (tiny ? 0x36800000u : 0x38000000u);
+  return __hiloint2double((int)((u & 0x80000000u) | (e ? ((u & 0x7fffffffu) >> 3) + bias : 0u)),
+                          (int)(u << 29));
+}
+
 // Cascaded (compensated) summation accumulator, Ogita-Rump-Oishi "Sum2":
 // the running sum is kept as hi + lo with every rounding error of hi
 // collected in lo.

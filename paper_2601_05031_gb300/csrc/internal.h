@@ -312,9 +312,9 @@ void launch_mu(Ctx& cx, const PhaseParams& P, const T* phi, T* g, T* mu, const S
 template <class T>
 void launch_source(Ctx& cx, const PhaseParams& P, const T* phi, const T* mu, Comp3<T> s_omega,
                    Comp3<T> f);
+// component c of v = v0 + curl psi' (v0: that component's table)
 template <class T>
-void launch_velocity(Ctx& cx, const PhaseParams& P, Comp3<T> psi, Comp3<T> psi_lo, Comp3<T> v0,
-                     Comp3<T> v);
+void launch_velocity(Ctx& cx, const PhaseParams& P, Comp3<T> psi, const T* v0, int c, T* v);
 // Diagnostic partial sums; out has kDiagQ doubles per block.
 constexpr int kDiagQ = 16;
 // vel_lo, om_lo, ps_lo: low words of the double-word velocity, omega' and
@@ -323,14 +323,19 @@ template <class T>
 void launch_diag(Ctx& cx, const PhaseParams& P, const T* phi, const T* phi_lo, const T* g,
                  const T* g_lo, Comp3<T> vel, Comp3<T> vel_lo, Comp3<T> omega, Comp3<T> om_lo,
                  Comp3<T> psi, Comp3<T> ps_lo, Comp3<const double> psi0_ring,
-                 Comp3<const double> v0d, T* sigma_t, double* partials, int nblocks, double* out);
+                 Comp3<const double> v0d, double* partials, int nblocks, double* out);
+// the in-plane stress sigma_t of a velocity as a field
 template <class T>
-void launch_stress_profile(Ctx& cx, const PhaseParams& P, Comp3<T> vel, Comp3<T> vel_lo,
+void launch_sigma_t(Ctx& cx, const PhaseParams& P, Comp3<T> vel, Comp3<T> vel_lo, T* out);
+// <sigma_xy>(y) from the x velocity; sums: scratch of ny nz doubles
+template <class T>
+void launch_stress_profile(Ctx& cx, const PhaseParams& P, const T* vx, const T* vx_lo, double* sums,
                            double* out);
-// Mixed path: v = v0 + curl psi' in FP64 from the double-word psi' and the
-// FP64 base-flow table, stored as a double word (v, v_lo).
+// Mixed path: component c of v = v0 + curl psi' from the double-word psi' and
+// the FP64 base-flow table: as a double word (v, v_lo), its high word alone
+// (v_lo null), or in FP64 (v64 not null).
 void launch_velocity_dw(Ctx& cx, const PhaseParams& P, Comp3<float> psi, Comp3<float> psi_lo,
-                        Comp3<const double> v0d, Comp3<float> v, Comp3<float> v_lo);
+                        const double* v0, int c, float* v, float* v_lo, double* v64 = nullptr);
 template <class Tin, class Tout>
 void launch_convert(Ctx& cx, const Tin* in, Tout* out, long long n);
 template <class T>

@@ -250,72 +250,126 @@ __global__ void k_source(PhaseParams P, const T* __restrict__ phi, const T* __re
 }
 
 // ---------------------------------------------------------------- velocity (eq. vecpot)
-// psi_lo (low words of a double-word psi', mixed path) may be null; the
-// difference of the double-word values is formed exactly before rounding.
+// One component of v = v0 + curl psi' per launch (a field export needs one
+// component, the observables ask for those they read).  Component c is
+// dA/da - dB/db with (A, a; B, b) = (psi_z, y; psi_y, z), (psi_x, z; psi_z, x),
+// (psi_y, x; psi_x, y).  Plain FP64 path:
 template <class T>
-__global__ void k_velocity(PhaseParams P, Comp3<T> psi, Comp3<T> psi_lo, Comp3<T> v0, Comp3<T> v) {
+__global__ void k_velocity(PhaseParams P, Comp3<T> psi, const T* __restrict__ v0, int c,
+                           T* __restrict__ v) {
   int i, j, k, comp_;
   if (!cell3(P.nx, P.ny, P.nz, i, j, k, comp_)) return;
-  const long long t = lin(i, j, k, P.nx, P.ny);
   const T hih = (T)(0.5 * P.inv_h);
-  PertView<T> X{psi.p[0], P.nx, P.ny, P.nz, P.zper};
-  PertView<T> Y{psi.p[1], P.nx, P.ny, P.nz, P.zper};
-  PertView<T> Z{psi.p[2], P.nx, P.ny, P.nz, P.zper};
-  const long long jk = j + (long long)k * P.ny;
-  if (psi_lo.p[0]) {
-    PertView<T> XL{psi_lo.p[0], P.nx, P.ny, P.nz, P.zper};
-    PertView<T> YL{psi_lo.p[1], P.nx, P.ny, P.nz, P.zper};
-    PertView<T> ZL{psi_lo.p[2], P.nx, P.ny, P.nz, P.zper};
-    // d(a)/dx with a = hi + lo: (a+ - a-) = (hi+ - hi-) + (lo+ - lo-)
-    auto d = [&](const PertView<T>& H, const PertView<T>& L, int i1, int j1, int k1, int i0, int j0,
-                 int k0) {
-      return ((H(i1, j1, k1) - H(i0, j0, k0)) + (L(i1, j1, k1) - L(i0, j0, k0))) * hih;
-    };
-    v.p[0][t] = v0.p[0][jk] + (d(Z, ZL, i, j + 1, k, i, j - 1, k) - d(Y, YL, i, j, k + 1, i, j, k - 1));
-    v.p[1][t] = v0.p[1][jk] + (d(X, XL, i, j, k + 1, i, j, k - 1) - d(Z, ZL, i + 1, j, k, i - 1, j, k));
-    v.p[2][t] = v0.p[2][jk] + (d(Y, YL, i + 1, j, k, i - 1, j, k) - d(X, XL, i, j + 1, k, i, j - 1, k));
-    return;
-  }
-  v.p[0][t] = v0.p[0][jk] + ((Z(i, j + 1, k) - Z(i, j - 1, k)) - (Y(i, j, k + 1) - Y(i, j, k - 1))) * hih;
-  v.p[1][t] = v0.p[1][jk] + ((X(i, j, k + 1) - X(i, j, k - 1)) - (Z(i + 1, j, k) - Z(i - 1, j, k))) * hih;
-  v.p[2][t] = v0.p[2][jk] + ((Y(i + 1, j, k) - Y(i - 1, j, k)) - (X(i, j + 1, k) - X(i, j - 1, k))) * hih;
+  PertView<T> A{psi.at(c == 0 ? 2 : c - 1), P.nx, P.ny, P.nz, P.zper};
+  PertView<T> B{psi.at(c == 2 ? 0 : c + 1), P.nx, P.ny, P.nz, P.zper};
+  const int ax = c == 2, ay = c == 0, az = c == 1;       // axis a
+  const int bx = c == 1, by = c == 2, bz = c == 0;       // axis b
+  v[lin(i, j, k, P.nx, P.ny)] =
+      v0[j + (long long)k * P.ny] +
+      ((A(i + ax, j + ay, k + az) - A(i - ax, j - ay, k - az)) -
+       (B(i + bx, j + by, k + bz) - B(i - bx, j - by, k - bz))) * hih;
 }
 
 // Velocity of the mixed path as a double word (hi + lo) for the observables
-// and FP64 exports: v = v0 + curl psi' formed in FP64 from the double-word
-// stream vector and the FP64 base-flow table, then split into its rounded
-// FP32 value and the FP32 rounding of the remainder (about 48 significant
-// bits).  Not on the time-stepping path.
-__global__ void k_velocity_dw(PhaseParams P, Comp3<float> psi, Comp3<float> psi_lo,
-                              Comp3<const double> v0d, Comp3<float> v, Comp3<float> v_lo) {
-  int i, j, k, comp_;
-  if (!cell3(P.nx, P.ny, P.nz, i, j, k, comp_)) return;
-  const long long t = lin(i, j, k, P.nx, P.ny);
-  const double hih = 0.5 * P.inv_h;
-  PertView<float> X{psi.p[0], P.nx, P.ny, P.nz, P.zper};
-  PertView<float> Y{psi.p[1], P.nx, P.ny, P.nz, P.zper};
-  PertView<float> Z{psi.p[2], P.nx, P.ny, P.nz, P.zper};
-  PertView<float> XL{psi_lo.p[0], P.nx, P.ny, P.nz, P.zper};
-  PertView<float> YL{psi_lo.p[1], P.nx, P.ny, P.nz, P.zper};
-  PertView<float> ZL{psi_lo.p[2], P.nx, P.ny, P.nz, P.zper};
-  auto d = [&](const PertView<float>& H, const PertView<float>& L, int i1, int j1, int k1, int i0,
-               int j0, int k0) {
-    return (((double)H(i1, j1, k1) + (double)L(i1, j1, k1)) -
-            ((double)H(i0, j0, k0) + (double)L(i0, j0, k0))) * hih;
-  };
-  const long long jk = j + (long long)k * P.ny;
-  double w[3];
-  w[0] = v0d.p[0][jk] + (d(Z, ZL, i, j + 1, k, i, j - 1, k) - d(Y, YL, i, j, k + 1, i, j, k - 1));
-  w[1] = v0d.p[1][jk] + (d(X, XL, i, j, k + 1, i, j, k - 1) - d(Z, ZL, i + 1, j, k, i - 1, j, k));
-  w[2] = v0d.p[2][jk] + (d(Y, YL, i + 1, j, k, i - 1, j, k) - d(X, XL, i, j + 1, k, i, j - 1, k));
-  for (int c = 0; c < 3; ++c) {
-    const float hi = __double2float_rn(w[c]);
-    v.at(c)[t] = hi;
-    v_lo.at(c)[t] = __double2float_rn(w[c] - (double)hi);
+// and the exports (not on the time-stepping path): v = v0 + ((a+ - a-) - (b+ -
+// b-)) / 2h from the double-word stream vector and the FP64 base-flow table.
+// FP64 units do two operations per clock and SM here, so the eight words are
+// summed by error-free FP32 transforms instead: high words, low words and the
+// errors of both as a three-word expansion, scaled by the words of 1 / 2h and
+// added to the three words of v0.  What is dropped is of order 2^-72 of the
+// operands; the result is v rounded to its two words, at least as close to the
+// real value as the FP64 evaluation it replaces (about 105 FP32 operations
+// instead of 22 FP64 ones; 492 -> 33 us for three components at
+// 256 x 128 x 128).
+struct VelScale {
+  float c1, c2, c3;   // 1 / 2h in three words
+};
+__device__ __forceinline__ void vel_dw(float aph, float apl, float amh, float aml, float bph, float bpl,
+                                       float bmh, float bml, VelScale C, float v1, float v2, float v3,
+                                       float& hi, float& lo) {
+  float s, s2, e1, e2, e3, t, t2, f1, f2, f3, g1, g2, g3;
+  two_sum(aph, -amh, s, e1);
+  two_sum(bmh, -bph, s2, e2);
+  two_sum(s, s2, s, e3);
+  two_sum(apl, -aml, t, f1);
+  two_sum(bml, -bpl, t2, f2);
+  two_sum(t, t2, t, f3);
+  two_sum(t, e1, t, g1);
+  two_sum(t, e2, t, g2);
+  two_sum(t, e3, t, g3);
+  float f = __fadd_rn(__fadd_rn(__fadd_rn(f1, f2), f3), __fadd_rn(__fadd_rn(g1, g2), g3));
+  // (s + t + f) (c1 + c2 + c3): leading words split exactly
+  const float p = __fmul_rn(s, C.c1), pe = __fmaf_rn(s, C.c1, -p);
+  float q = __fmul_rn(t, C.c1);
+  f = __fmaf_rn(f, C.c1, __fmaf_rn(t, C.c1, -q));
+  two_sum(q, pe, q, g1);
+  f = __fadd_rn(f, g1);
+  if (C.c2 != 0.f || C.c3 != 0.f) {
+    const float r = __fmul_rn(s, C.c2);
+    two_sum(q, r, q, g1);
+    f = __fadd_rn(f, __fadd_rn(g1, __fmaf_rn(s, C.c2, -r)));
+    f = __fmaf_rn(s, C.c3, __fmaf_rn(t, C.c2, f));
+  }
+  float u, w;
+  two_sum(p, v1, u, w);
+  two_sum(w, q, w, g1);
+  two_sum(w, v2, w, g2);
+  f = __fadd_rn(f, __fadd_rn(__fadd_rn(g1, g2), v3));
+  two_sum(u, w, u, w);
+  two_sum(w, f, w, f);
+  const FF r = fast_two_sum(u, w);
+  hi = r.hi;
+  lo = __fadd_rn(r.lo, f);
+  // the transforms turn an infinity into NaN: keep it in the high word
+  const float plain = v1 + ((aph - amh) - (bph - bmh)) * C.c1;
+  if (!isfinite(plain)) {
+    hi = plain;
+    lo = plain - plain;
   }
 }
 
+__device__ __forceinline__ void split3(double v, float& a, float& b, float& c) {
+  a = __double2float_rn(v);
+  const double r = v - (double)a;
+  b = __double2float_rn(r);
+  c = __double2float_rn(r - (double)b);
+}
+
+// What the kernel writes: the two words (f, f_lo), the high word alone into a
+// caller's FP32 field, or their sum into a caller's FP64 field.
+enum { kVelWords = 0, kVelF32 = 1, kVelF64 = 2 };
+
+template <int C, int OUT>
+__global__ void k_velocity_dw(PhaseParams P, const float* __restrict__ ah, const float* __restrict__ al,
+                              const float* __restrict__ bh, const float* __restrict__ bl,
+                              const double* __restrict__ v0, VelScale S, float* __restrict__ vh,
+                              float* __restrict__ vl, double* __restrict__ vd) {
+  int i, j, k, comp_;
+  if (!cell3(P.nx, P.ny, P.nz, i, j, k, comp_)) return;
+  PertView<float> A{ah, P.nx, P.ny, P.nz, P.zper}, AL{al, P.nx, P.ny, P.nz, P.zper};
+  PertView<float> B{bh, P.nx, P.ny, P.nz, P.zper}, BL{bl, P.nx, P.ny, P.nz, P.zper};
+  constexpr int ax = C == 2, ay = C == 0, az = C == 1, bx = C == 1, by = C == 2, bz = C == 0;
+  float v1, v2, v3, hi, lo;
+  split3(v0[j + (long long)k * P.ny], v1, v2, v3);
+  vel_dw(A(i + ax, j + ay, k + az), AL(i + ax, j + ay, k + az), A(i - ax, j - ay, k - az),
+         AL(i - ax, j - ay, k - az), B(i + bx, j + by, k + bz), BL(i + bx, j + by, k + bz),
+         B(i - bx, j - by, k - bz), BL(i - bx, j - by, k - bz), S, v1, v2, v3, hi, lo);
+  const long long t = lin(i, j, k, P.nx, P.ny);
+  if (OUT != kVelF64) vh[t] = hi;
+  if (OUT == kVelWords) vl[t] = lo;
+  if (OUT == kVelF64) vd[t] = (double)hi + (double)lo;
+}
+
 // ---------------------------------------------------------------- observables
+// A field value in FP64 (lo: the low word of a double word on the mixed path).
+__device__ __forceinline__ double val64(const double* __restrict__ a, const double*, long long t) {
+  return a[t];
+}
+__device__ __forceinline__ double val64(const float* __restrict__ a, const float* __restrict__ lo,
+                                        long long t) {
+  return lo ? f2d(a[t]) + f2d(lo[t]) : f2d(a[t]);
+}
+
 // Velocity (materialised; lo: the low words of a double-word velocity, or
 // null) with the no-slip wall velocity on the wall nodes.
 template <class T>
@@ -331,19 +385,7 @@ struct VelView {
     if (j >= ny) return P->vwall[1][comp];
     if (k < 0) return P->vwall[2][comp];
     if (k >= nz) return P->vwall[3][comp];
-    const long long t = lin(i, j, k, nx, ny);
-    return lo ? (double)a[t] + (double)lo[t] : (double)a[t];
-  }
-};
-
-// A double-word perturbation field (hi + lo; lo may be null) read in FP64,
-// zero on the wall nodes.
-template <class T>
-struct PertView2 {
-  PertView<T> hi, lo;
-  bool has_lo;
-  __device__ __forceinline__ double operator()(int i, int j, int k) const {
-    return has_lo ? (double)hi(i, j, k) + (double)lo(i, j, k) : (double)hi(i, j, k);
+    return val64(a, lo, lin(i, j, k, nx, ny));
   }
 };
 
@@ -362,165 +404,278 @@ struct V0View {
   }
 };
 
+// |x| as an integer that orders like it (0 for a NaN, which fmax skips too)
+__device__ __forceinline__ long long abs_bits(double x) {
+  const long long b = __double_as_longlong(x) & 0x7fffffffffffffffLL;
+  return b <= 0x7ff0000000000000LL ? b : 0;
+}
+
 // q: 0 dissipation integrand, 1 body-free dissipation integrand, 2 |omega'|^2,
 // 3 |psi'|^2, 4 w = (1-phi)/2, 5..7 w x, w y, w z, 8 energy density,
 // 9 max |div v|, 10 max |div psi|, 11 max sigma_t, 12 (Helfrich with a
 // membrane tension) the face-difference area density over c_A / eps.
 // vel_lo, om_lo, ps_lo: low words of double-word velocity, omega' and psi'
-// (mixed path), or null pointers.
+// (mixed path), or null pointers.  Two kernels: the velocity's quantities
+// (0, 1, 9, 11), and the others.
+//
+// Bound by the FP64 units (two operations per clock and SM, long latency):
+// conversions go through f2d, the strain is taken from raw differences (its
+// scale 1 / 2h, the viscosity and h are applied once per block), each
+// symmetric pair once, maxima compare bits, the one square root is taken of
+// the maximum, and what does not depend on x is done once per row (a warp
+// takes whole rows).  About 80 FP64 operations per cell instead of 270:
+// 2,114 -> 406 + 326 us at 256 x 128 x 128 (470 G operations/s; additions alone
+// reach 490 here).
 template <class T>
-__global__ void k_diag(PhaseParams P, const T* __restrict__ phi, const T* __restrict__ phi_lo,
-                       const T* __restrict__ g, const T* __restrict__ g_lo, Comp3<T> vel,
-                       Comp3<T> vel_lo, Comp3<T> omega, Comp3<T> om_lo, Comp3<T> psi,
-                       Comp3<T> ps_lo, Comp3<const double> psi0r, Comp3<const double> v0d,
-                       T* sigma_t, double* partials) {
-  double q[kDiagQ];
-  for (int a = 0; a < kDiagQ; ++a) q[a] = 0.0;
-  const double hih = 0.5 * P.inv_h, eta = 1.0 / P.inv_eta, h = P.h;
-  const int ny2 = P.ny + 2;
-  for (int row = blockIdx.x; row < P.ny * P.nz; row += gridDim.x) {
-   const int j = row % P.ny, k = row / P.ny;
-   for (int i = threadIdx.x; i < P.nx; i += blockDim.x) {
-    const long long t = lin(i, j, k, P.nx, P.ny);
-    double G[3][3], G0[3][3];
-    for (int c = 0; c < 3; ++c) {
-      VelView<T> V{vel.p[c], vel_lo.p[c], P.nx, P.ny, P.nz, P.zper, c, &P};
-      G[c][0] = (V(i + 1, j, k) - V(i - 1, j, k)) * hih;
-      G[c][1] = (V(i, j + 1, k) - V(i, j - 1, k)) * hih;
-      G[c][2] = (V(i, j, k + 1) - V(i, j, k - 1)) * hih;
-      V0View W{v0d.p[c], P.ny, P.nz, P.zper, c, &P};
-      G0[c][0] = 0.0;
-      G0[c][1] = (W(j + 1, k) - W(j - 1, k)) * hih;
-      G0[c][2] = (W(j, k + 1) - W(j, k - 1)) * hih;
-    }
-    double d = 0.0, d0 = 0.0;
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        const double e = G[a][b] + G[b][a], e0 = G0[a][b] + G0[b][a];
-        d += e * e;
-        d0 += e0 * e0;
+__global__ void __launch_bounds__(kBlock, 4)
+k_diag_flow(PhaseParams P, Comp3<T> vel, Comp3<T> vel_lo, Comp3<const double> v0d, double* partials) {
+  double diss = 0.0, diss0 = 0.0;
+  long long mv = 0, ms = 0;   // maxima of |div v| and of the squared shears
+  const double hih = 0.5 * P.inv_h, eta = 1.0 / P.inv_eta;
+  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < P.ny * P.nz; row += gridDim.x * wpb) {
+    const int k = row / P.ny, j = row - k * P.ny;
+    if (lane == 0) {   // the body-free flow does not depend on x
+      double G0[3][3];
+      for (int c = 0; c < 3; ++c) {
+        V0View W{v0d.p[c], P.ny, P.nz, P.zper, c, &P};
+        G0[c][0] = 0.0;
+        G0[c][1] = W(j + 1, k) - W(j - 1, k);
+        G0[c][2] = W(j, k + 1) - W(j, k - 1);
       }
-    q[0] += d;
-    q[1] += d0;
-    double o2 = 0.0, p2 = 0.0;
-    for (int c = 0; c < 3; ++c) {
-      const double o = (double)omega.p[c][t] + (om_lo.p[c] ? (double)om_lo.p[c][t] : 0.0);
-      const double p = (double)psi.p[c][t] + (ps_lo.p[c] ? (double)ps_lo.p[c][t] : 0.0);
-      o2 += o * o;
-      p2 += p * p;
+      double d0 = 0.0;
+      for (int a = 0; a < 3; ++a)
+        for (int b = 0; b < 3; ++b) {
+          const double e0 = G0[a][b] + G0[b][a];
+          d0 += e0 * e0;
+        }
+      diss0 += d0 * (double)P.nx;
     }
-    q[2] += o2;
-    q[3] += p2;
-    const double f = (double)phi[t] + (phi_lo ? (double)phi_lo[t] : 0.0);
-    const double w = 0.5 * (1.0 - f);
-    q[4] += w;
-    q[5] += w * (i + 0.5) * h;
-    q[6] += w * (j + 1.0) * h;
-    q[7] += w * (P.zper ? (k + 0.5) : (k + 1.0)) * h;
-    if (P.fe_kind == VSV_HELFRICH) {
-      const double gg = (double)g[t] + (g_lo ? (double)g_lo[t] : 0.0);
-      q[8] += gg * gg;
-      if (P.beta_t != 0.0) {   // membrane tension: the face-difference area density
+    // rows of the six neighbours' kinds (negative: a wall, whose index is kept)
+    const int km = P.zper ? wrap_idx(k - 1, P.nz) : k - 1, kp = P.zper ? wrap_idx(k + 1, P.nz) : k + 1;
+    const long long rc = (long long)row * P.nx, ps = (long long)P.ny * P.nx;
+    const long long rym = j > 0 ? rc - P.nx : -1, ryp = j < P.ny - 1 ? rc + P.nx : -2;
+    const long long rzm = km >= 0 ? rc + (km - k) * ps : -3, rzp = kp < P.nz ? rc + (kp - k) * ps : -4;
+    auto v = [&](int c, long long r, int i) {
+      return r >= 0 ? val64(vel.at(c), vel_lo.at(c), r + i) : P.vwall[-1 - r][c];
+    };
+    for (int i = lane; i < P.nx; i += 32) {
+      const int il = i > 0 ? i - 1 : P.nx - 1, ir = i < P.nx - 1 ? i + 1 : 0;
+      // raw central differences
+      const double xx = v(0, rc, ir) - v(0, rc, il);
+      const double yy = v(1, ryp, i) - v(1, rym, i);
+      const double zz = v(2, rzp, i) - v(2, rzm, i);
+      const double xy = (v(0, ryp, i) - v(0, rym, i)) + (v(1, rc, ir) - v(1, rc, il));
+      const double yz = (v(1, rzp, i) - v(1, rzm, i)) + (v(2, ryp, i) - v(2, rym, i));
+      const double xz = (v(0, rzp, i) - v(0, rzm, i)) + (v(2, rc, ir) - v(2, rc, il));
+      const double dg = xx * xx + yy * yy + zz * zz, sh = xy * xy + yz * yz + xz * xz;
+      diss += 2.0 * dg + sh;          // half of sum_ij (2 e_ij)^2
+      ms = max(ms, abs_bits(sh));
+      mv = max(mv, abs_bits(xx + yy + zz));
+    }
+  }
+  diss = block_sum(diss * (2.0 * hih * hih));
+  diss0 = block_sum(diss0 * (hih * hih));
+  const double dv = block_max(__longlong_as_double(mv) * hih);
+  const double st = block_max(eta * hih * sqrt(__longlong_as_double(ms)));
+  if (threadIdx.x == 0) {
+    double* out = partials + (long long)blockIdx.x * kDiagQ;
+    out[0] = diss;
+    out[1] = diss0;
+    out[9] = dv;
+    out[11] = st;
+  }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kBlock, 4)
+k_diag_state(PhaseParams P, const T* __restrict__ phi, const T* __restrict__ phi_lo,
+             const T* __restrict__ g, const T* __restrict__ g_lo, Comp3<T> omega, Comp3<T> om_lo,
+             Comp3<T> psi, Comp3<T> ps_lo, Comp3<const double> psi0r, double* partials) {
+  double q[7], q12 = 0.0;   // quantities 2 .. 8
+  for (int a = 0; a < 7; ++a) q[a] = 0.0;
+  long long mp = 0;         // maximum of |div psi|
+  const double hih = 0.5 * P.inv_h, h = P.h;
+  const bool tension = P.fe_kind == VSV_HELFRICH && P.beta_t != 0.0;
+  const int ny2 = P.ny + 2, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < P.ny * P.nz; row += gridDim.x * wpb) {
+    const int k = row / P.ny, j = row - k * P.ny;
+    const int km = P.zper ? wrap_idx(k - 1, P.nz) : k - 1, kp = P.zper ? wrap_idx(k + 1, P.nz) : k + 1;
+    const long long rc = (long long)row * P.nx, ps = (long long)P.ny * P.nx;
+    const long long rym = j > 0 ? rc - P.nx : -1, ryp = j < P.ny - 1 ? rc + P.nx : -1;
+    const long long rzm = km >= 0 ? rc + (km - k) * ps : -1, rzp = kp < P.nz ? rc + (kp - k) * ps : -1;
+    // div psi with psi = psi0(y, z) + psi'; psi0 ring table holds the wall data
+    auto r0 = [&](int c, int jj, int kk) { return psi0r.p[c][(jj + 1) + (long long)(kk + 1) * ny2]; };
+    const double div0 = (r0(1, j + 1, k) - r0(1, j - 1, k)) + (r0(2, j, kp) - r0(2, j, km));
+    auto p = [&](int c, long long r, int i) {
+      return r >= 0 ? val64(psi.at(c), ps_lo.at(c), r + i) : 0.0;
+    };
+    double wr = 0.0;
+    for (int i = lane; i < P.nx; i += 32) {
+      const int il = i > 0 ? i - 1 : P.nx - 1, ir = i < P.nx - 1 ? i + 1 : 0;
+      const long long t = rc + i;
+      mp = max(mp, abs_bits((p(0, rc, ir) - p(0, rc, il)) + (p(1, ryp, i) - p(1, rym, i)) +
+                            (p(2, rzp, i) - p(2, rzm, i)) + div0));
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const double o = val64(omega.at(c), om_lo.at(c), t), s = val64(psi.at(c), ps_lo.at(c), t);
+        q[0] += o * o;
+        q[1] += s * s;
+      }
+      const double f = val64(phi, phi_lo, t);
+      const double w = 0.5 - 0.5 * f;
+      wr += w;
+      q[3] += w * f2d((float)i + 0.5f);
+      if (P.fe_kind == VSV_HELFRICH) {
+        const double gg = val64(g, g_lo, t);
+        q[6] += gg * gg;
+        if (tension) {   // the face-difference area density
+          ScalarView<T> F{phi, P.nx, P.ny, P.nz, P.zper};
+          ScalarView<T> FL{phi_lo ? phi_lo : phi, P.nx, P.ny, P.nz, P.zper};
+          auto val = [&](int ii, int jj, int kk) {
+            return (double)F(ii, jj, kk) + (phi_lo ? (double)FL(ii, jj, kk) : 0.0);
+          };
+          const double dx = (val(i + 1, j, k) - f) * P.inv_h;
+          double faces = dx * dx;
+          if (j + 1 < P.ny) {
+            const double dy = (val(i, j + 1, k) - f) * P.inv_h;
+            faces += dy * dy;
+          }
+          if (P.zper || k + 1 < P.nz) {
+            const double dz = (val(i, j, k + 1) - f) * P.inv_h;
+            faces += dz * dz;
+          }
+          q12 += 0.25 * (f * f - 1.0) * (f * f - 1.0) + 0.5 * P.eps * P.eps * faces;
+        }
+      } else {
         ScalarView<T> F{phi, P.nx, P.ny, P.nz, P.zper};
-        ScalarView<T> FL{phi_lo ? phi_lo : phi, P.nx, P.ny, P.nz, P.zper};
-        auto val = [&](int ii, int jj, int kk) {
-          return (double)F(ii, jj, kk) + (phi_lo ? (double)FL(ii, jj, kk) : 0.0);
-        };
-        const double dx = (val(i + 1, j, k) - f) * P.inv_h;
+        double e = 0.25 * (f * f - 1.0) * (f * f - 1.0);
+        const double dx = ((double)F(i + 1, j, k) - f) * P.inv_h;
         double faces = dx * dx;
         if (j + 1 < P.ny) {
-          const double dy = (val(i, j + 1, k) - f) * P.inv_h;
+          const double dy = ((double)F(i, j + 1, k) - f) * P.inv_h;
           faces += dy * dy;
         }
         if (P.zper || k + 1 < P.nz) {
-          const double dz = (val(i, j, k + 1) - f) * P.inv_h;
+          const double dz = ((double)F(i, j, k + 1) - f) * P.inv_h;
           faces += dz * dz;
         }
-        q[12] += 0.25 * (f * f - 1.0) * (f * f - 1.0) + 0.5 * P.eps * P.eps * faces;
+        q[6] += e + 0.5 * P.sigma * faces;
       }
-    } else {
-      ScalarView<T> F{phi, P.nx, P.ny, P.nz, P.zper};
-      double e = 0.25 * (f * f - 1.0) * (f * f - 1.0);
-      const double dx = ((double)F(i + 1, j, k) - f) * P.inv_h;
-      double faces = dx * dx;
-      if (j + 1 < P.ny) {
-        const double dy = ((double)F(i, j + 1, k) - f) * P.inv_h;
-        faces += dy * dy;
-      }
-      if (P.zper || k + 1 < P.nz) {
-        const double dz = ((double)F(i, j, k + 1) - f) * P.inv_h;
-        faces += dz * dz;
-      }
-      q[8] += e + 0.5 * P.sigma * faces;
     }
-    q[9] = fmax(q[9], fabs(G[0][0] + G[1][1] + G[2][2]));
-    // div psi with psi = psi0(y, z) + psi'; psi0 ring table holds the wall data
-    const bool pl = ps_lo.p[0] != nullptr;
-    PertView2<T> PX{{psi.p[0], P.nx, P.ny, P.nz, P.zper}, {pl ? ps_lo.p[0] : psi.p[0], P.nx, P.ny, P.nz, P.zper}, pl};
-    PertView2<T> PY{{psi.p[1], P.nx, P.ny, P.nz, P.zper}, {pl ? ps_lo.p[1] : psi.p[1], P.nx, P.ny, P.nz, P.zper}, pl};
-    PertView2<T> PZ{{psi.p[2], P.nx, P.ny, P.nz, P.zper}, {pl ? ps_lo.p[2] : psi.p[2], P.nx, P.ny, P.nz, P.zper}, pl};
-    auto r0 = [&](int c, int jj, int kk) -> double {
-      if (P.zper) kk = wrap_idx(kk, P.nz);
-      return psi0r.p[c][(jj + 1) + (long long)(kk + 1) * ny2];
-    };
-    const double dpx = (PX(i + 1, j, k) - PX(i - 1, j, k)) * hih;
-    const double dpy = (PY(i, j + 1, k) - PY(i, j - 1, k) + r0(1, j + 1, k) -
-                        r0(1, j - 1, k)) * hih;
-    const double dpz = (PZ(i, j, k + 1) - PZ(i, j, k - 1) + r0(2, j, k + 1) -
-                        r0(2, j, k - 1)) * hih;
-    q[10] = fmax(q[10], fabs(dpx + dpy + dpz));
-    const double sxy = eta * (G[0][1] + G[1][0]);
-    const double syz = eta * (G[1][2] + G[2][1]);
-    const double sxz = eta * (G[0][2] + G[2][0]);
-    const double st = sqrt(sxy * sxy + syz * syz + sxz * sxz);
-    q[11] = fmax(q[11], st);
-    if (sigma_t) sigma_t[t] = (T)st;
-   }
+    q[2] += wr;
+    q[4] += wr * (j + 1.0);
+    q[5] += wr * (P.zper ? (k + 0.5) : (k + 1.0));
   }
-  for (int a = 0; a < 9; ++a) {
+  q[3] *= h; q[4] *= h; q[5] *= h;
+  double* out = partials + (long long)blockIdx.x * kDiagQ;
+  for (int a = 0; a < 7; ++a) {
     const double s = block_sum(q[a]);
-    if (threadIdx.x == 0) partials[(long long)blockIdx.x * kDiagQ + a] = s;
+    if (threadIdx.x == 0) out[2 + a] = s;
   }
-  for (int a = 9; a < 12; ++a) {
-    const double s = block_max(q[a]);
-    if (threadIdx.x == 0) partials[(long long)blockIdx.x * kDiagQ + a] = s;
-  }
-  {
-    const double s = block_sum(q[12]);
-    if (threadIdx.x == 0) partials[(long long)blockIdx.x * kDiagQ + 12] = s;
+  const double m = block_max(__longlong_as_double(mp) * hih), s12 = block_sum(q12);
+  if (threadIdx.x == 0) {
+    out[10] = m;
+    out[12] = s12;
   }
 }
 
-__global__ void k_diag_finalize(const double* partials, int nblocks, double* out) {
-  for (int a = 0; a < 13; ++a) {   // 0..8 and 12 are sums, 9..11 maxima
-    const bool sum = a < 9 || a == 12;
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-      const double v = partials[(long long)b * kDiagQ + a];
-      s = sum ? s + v : fmax(s, v);
+// The in-plane stress sigma_t = eta sqrt((2 e_xy)^2 + (2 e_yz)^2 + (2 e_xz)^2)
+// as a field.  FP64 path; and mixed path, stored in FP32, from double words in
+// FP32 arithmetic (relative error of a few 2^-44 before the one rounding, the
+// root corrected by its remainder), clear of the FP64 units (88 us at
+// 256 x 128 x 128; as one of the diagnostics' outputs 2,114).
+__global__ void k_sigma_t(PhaseParams P, Comp3<double> vel, double* __restrict__ out) {
+  int i, j, k, comp_;
+  if (!cell3(P.nx, P.ny, P.nz, i, j, k, comp_)) return;
+  VelView<double> X{vel.p[0], nullptr, P.nx, P.ny, P.nz, P.zper, 0, &P};
+  VelView<double> Y{vel.p[1], nullptr, P.nx, P.ny, P.nz, P.zper, 1, &P};
+  VelView<double> Z{vel.p[2], nullptr, P.nx, P.ny, P.nz, P.zper, 2, &P};
+  const double f = 0.5 * P.inv_h / P.inv_eta;
+  const double xy = (X(i, j + 1, k) - X(i, j - 1, k)) + (Y(i + 1, j, k) - Y(i - 1, j, k));
+  const double yz = (Y(i, j, k + 1) - Y(i, j, k - 1)) + (Z(i, j + 1, k) - Z(i, j - 1, k));
+  const double xz = (X(i, j, k + 1) - X(i, j, k - 1)) + (Z(i + 1, j, k) - Z(i - 1, j, k));
+  out[lin(i, j, k, P.nx, P.ny)] = f * sqrt(xy * xy + yz * yz + xz * xz);
+}
+__global__ void k_sigma_t_dw(PhaseParams P, Comp3<float> vel, Comp3<float> vel_lo, FF f2,
+                             float* __restrict__ out) {
+  int i, j, k, comp_;
+  if (!cell3(P.nx, P.ny, P.nz, i, j, k, comp_)) return;
+  auto v = [&](int c, int ii, int jj, int kk) {
+    ii = wrap_idx(ii, P.nx);
+    if (P.zper) kk = wrap_idx(kk, P.nz);
+    const int w = jj < 0 ? 0 : (jj >= P.ny ? 1 : (kk < 0 ? 2 : (kk >= P.nz ? 3 : -1)));
+    if (w >= 0) {
+      const double b = P.vwall[w][c];
+      const float hi = (float)b;
+      return FF{hi, (float)(b - (double)hi)};
     }
-    s = sum ? block_sum(s) : block_max(s);
-    if (threadIdx.x == 0) out[a] = s;
-  }
+    const long long t = lin(ii, jj, kk, P.nx, P.ny);
+    return FF{vel.at(c)[t], vel_lo.at(c)[t]};
+  };
+  auto shear = [&](FF ap, FF am, FF bp, FF bm) {
+    const FF s = ff_add(ff_add(ap, ff_neg(am)), ff_add(bp, ff_neg(bm)));
+    return ff_mul(s, s);
+  };
+  FF s = shear(v(0, i, j + 1, k), v(0, i, j - 1, k), v(1, i + 1, j, k), v(1, i - 1, j, k));
+  s = ff_add(s, shear(v(1, i, j, k + 1), v(1, i, j, k - 1), v(2, i, j + 1, k), v(2, i, j - 1, k)));
+  s = ff_add(s, shear(v(0, i, j, k + 1), v(0, i, j, k - 1), v(2, i + 1, j, k), v(2, i - 1, j, k)));
+  s = ff_mul(s, f2);
+  float r = sqrtf(s.hi);
+  if (r > 0.f && isfinite(r)) r += (__fmaf_rn(-r, r, s.hi) + s.lo) / (2.f * r);
+  out[lin(i, j, k, P.nx, P.ny)] = r;
 }
 
-// <sigma_xy>(y): one block per y row, fixed-order sum over x and z.
-template <class T>
-__global__ void k_stress_profile(PhaseParams P, Comp3<T> vel, Comp3<T> vel_lo, double* out) {
-  const int j = blockIdx.x;
-  const double hih = 0.5 * P.inv_h, eta = 1.0 / P.inv_eta;
-  VelView<T> VX{vel.p[0], vel_lo.p[0], P.nx, P.ny, P.nz, P.zper, 0, &P};
-  VelView<T> VY{vel.p[1], vel_lo.p[1], P.nx, P.ny, P.nz, P.zper, 1, &P};
+// one block per quantity
+__global__ void k_diag_finalize(const double* partials, int nblocks, double* out) {
+  const int a = blockIdx.x;   // 0..8 and 12 are sums, 9..11 maxima
+  const bool sum = a < 9 || a == 12;
   double s = 0.0;
-  const long long m = (long long)P.nx * P.nz;
-  for (long long t = threadIdx.x; t < m; t += blockDim.x) {
-    const int i = (int)(t % P.nx), k = (int)(t / P.nx);
-    const double dvx_dy = (VX(i, j + 1, k) - VX(i, j - 1, k)) * hih;
-    const double dvy_dx = (VY(i + 1, j, k) - VY(i - 1, j, k)) * hih;
-    s += eta * (dvx_dy + dvy_dx);
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
+    const double v = partials[(long long)b * kDiagQ + a];
+    s = sum ? s + v : fmax(s, v);
   }
+  s = sum ? block_sum(s) : block_max(s);
+  if (threadIdx.x == 0) out[a] = s;
+}
+
+// <sigma_xy>(y) = eta <d_y v_x + d_x v_y> over x and z.  The mean of the
+// periodic central difference d_x v_y vanishes term by term, and that of
+// d_y v_x is the central difference of the row means of v_x: one pass that
+// sums v_x over each row of a chunk of planes (double words in cascaded sums),
+// then the differences (308 -> 14 + 4 us at 256 x 128 x 128).
+template <class T>
+__global__ void k_row_sums(PhaseParams P, const T* __restrict__ vx, const T* __restrict__ vx_lo,
+                           int kchunk, double* sums) {
+  const int j = blockIdx.x, kb = blockIdx.y * kchunk, ke = min(kb + kchunk, P.nz);
+  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  double s = 0.0;
+  CascadeSum cs(0.f);
+  for (int k = kb + (threadIdx.x >> 5); k < ke; k += wpb)
+    for (int i = lane; i < P.nx; i += 32) {
+      const long long t = lin(i, j, k, P.nx, P.ny);
+      if constexpr (sizeof(T) == 4) {
+        cs.add(vx[t]);
+        cs.add(vx_lo[t]);
+      } else {
+        s += vx[t];
+      }
+    }
+  if constexpr (sizeof(T) == 4) s = (double)cs.hi + (double)cs.lo;
   s = block_sum(s);
-  if (threadIdx.x == 0) out[j] = s / (double)m;
+  if (threadIdx.x == 0) sums[(long long)blockIdx.y * P.ny + j] = s;
+}
+__global__ void k_stress_profile(PhaseParams P, const double* sums, int chunks, double* out) {
+  const double m = (double)P.nx * (double)P.nz, eta = 1.0 / P.inv_eta;
+  auto row = [&](int j) {
+    if (j < 0) return m * P.vwall[0][0];
+    if (j >= P.ny) return m * P.vwall[1][0];
+    double s = 0.0;
+    for (int c = 0; c < chunks; ++c) s += sums[(long long)c * P.ny + j];
+    return s;
+  };
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < P.ny; j += gridDim.x * blockDim.x)
+    out[j] = eta * ((row(j + 1) - row(j - 1)) * (0.5 * P.inv_h)) / m;
 }
 
 // ---------------------------------------------------------------- small utilities
@@ -991,6 +1146,56 @@ __device__ __forceinline__ bool cell4(const PhaseParams& P, int& i0, int& j, int
 
 }  // namespace
 
+// k_velocity_dw on 4-cell groups
+template <int C, int OUT>
+__global__ void __launch_bounds__(256) k_velocity_dw4(PhaseParams P, const float* __restrict__ ah,
+                                                      const float* __restrict__ al,
+                                                      const float* __restrict__ bh,
+                                                      const float* __restrict__ bl,
+                                                      const double* __restrict__ v0, VelScale S,
+                                                      float* __restrict__ vh, float* __restrict__ vl,
+                                                      double* __restrict__ vd) {
+  int i0, j, k;
+  if (!cell4(P, i0, j, k)) return;
+  const Geo4 G = geo4(P, i0, j, k, true);
+  float v1, v2, v3;
+  split3(v0[j + (long long)k * P.ny], v1, v2, v3);
+  // plus and minus neighbours along axis D of the four cells
+  auto pm = [&](const float* __restrict__ a, int axis, float4& p, float4& m) {
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (axis == 0) {
+      const float4 c = ld4g(a + G.rc + i0);
+      p = make_float4(c.y, c.z, c.w, a[G.rc + G.ir]);
+      m = make_float4(a[G.rc + G.il], c.x, c.y, c.z);
+    } else if (axis == 1) {
+      p = G.ryp >= 0 ? ld4g(a + G.ryp + i0) : z;
+      m = G.rym >= 0 ? ld4g(a + G.rym + i0) : z;
+    } else {
+      p = G.rzp >= 0 ? ld4g(a + G.rzp + i0) : z;
+      m = G.rzm >= 0 ? ld4g(a + G.rzm + i0) : z;
+    }
+  };
+  constexpr int aa = C == 2 ? 0 : (C == 0 ? 1 : 2), ab = C == 1 ? 0 : (C == 2 ? 1 : 2);
+  float4 aph, amh, apl, aml, bph, bmh, bpl, bml;
+  pm(ah, aa, aph, amh);
+  pm(al, aa, apl, aml);
+  pm(bh, ab, bph, bmh);
+  pm(bl, ab, bpl, bml);
+  float h[4], l[4];
+#pragma unroll
+  for (int o = 0; o < 4; ++o)
+    vel_dw(e4(aph, o), e4(apl, o), e4(amh, o), e4(aml, o), e4(bph, o), e4(bpl, o), e4(bmh, o),
+           e4(bml, o), S, v1, v2, v3, h[o], l[o]);
+  const long long t = G.rc + i0;
+  if (OUT != kVelF64) *reinterpret_cast<float4*>(vh + t) = make_float4(h[0], h[1], h[2], h[3]);
+  if (OUT == kVelWords) *reinterpret_cast<float4*>(vl + t) = make_float4(l[0], l[1], l[2], l[3]);
+  if (OUT == kVelF64) {
+    double2* d = reinterpret_cast<double2*>(vd + t);
+    d[0] = make_double2((double)h[0] + (double)l[0], (double)h[1] + (double)l[1]);
+    d[1] = make_double2((double)h[2] + (double)l[2], (double)h[3] + (double)l[3]);
+  }
+}
+
 __global__ void __launch_bounds__(256, 3) k_phi_update_ff4(PhaseParams P, const float* __restrict__ phi,
                                  const float* __restrict__ phi_lo, const float* __restrict__ mu,
                                  Comp3<float> psi, Comp3<float> v0, Scalars* S, float dt,
@@ -1372,18 +1577,44 @@ void launch_source(Ctx& cx, const PhaseParams& P, const T* phi, const T* mu, Com
 }
 
 template <class T>
-void launch_velocity(Ctx& cx, const PhaseParams& P, Comp3<T> psi, Comp3<T> psi_lo, Comp3<T> v0,
-                     Comp3<T> v) {
+void launch_velocity(Ctx& cx, const PhaseParams& P, Comp3<T> psi, const T* v0, int c, T* v) {
   cx.before(-1);
-  k_velocity<T><<<grid3(P.nx, P.ny, P.nz, 1), block3(), 0, cx.stream>>>(P, psi, psi_lo, v0, v);
+  k_velocity<T><<<grid3(P.nx, P.ny, P.nz, 1), block3(), 0, cx.stream>>>(P, psi, v0, c, v);
   cx.after(-1);
 }
 
+namespace {
+template <int C, int OUT>
+void velocity_dw(Ctx& cx, const PhaseParams& P, Comp3<float> psi, Comp3<float> psi_lo, const double* v0,
+                 float* v, float* v_lo, double* vd) {
+  constexpr int A = C == 0 ? 2 : C - 1, B = C == 2 ? 0 : C + 1;
+  const double hih = 0.5 * P.inv_h;
+  VelScale S;
+  S.c1 = (float)hih;
+  S.c2 = (float)(hih - (double)S.c1);
+  S.c3 = (float)(hih - (double)S.c1 - (double)S.c2);
+  const float *ah = psi.p[A], *al = psi_lo.p[A], *bh = psi.p[B], *bl = psi_lo.p[B];
+  if (use4(P) && aligned16(v) && aligned16(v_lo) && aligned16(vd))
+    k_velocity_dw4<C, OUT><<<grid4(P), dim3(32, 8), 0, cx.stream>>>(P, ah, al, bh, bl, v0, S, v, v_lo, vd);
+  else
+    k_velocity_dw<C, OUT><<<grid3(P.nx, P.ny, P.nz, 1), block3(), 0, cx.stream>>>(P, ah, al, bh, bl, v0, S,
+                                                                               v, v_lo, vd);
+}
+template <int OUT>
+void velocity_dw_c(Ctx& cx, const PhaseParams& P, Comp3<float> psi, Comp3<float> psi_lo, const double* v0,
+                   int c, float* v, float* v_lo, double* vd) {
+  if (c == 0) velocity_dw<0, OUT>(cx, P, psi, psi_lo, v0, v, v_lo, vd);
+  else if (c == 1) velocity_dw<1, OUT>(cx, P, psi, psi_lo, v0, v, v_lo, vd);
+  else velocity_dw<2, OUT>(cx, P, psi, psi_lo, v0, v, v_lo, vd);
+}
+}  // namespace
+
 void launch_velocity_dw(Ctx& cx, const PhaseParams& P, Comp3<float> psi, Comp3<float> psi_lo,
-                        Comp3<const double> v0d, Comp3<float> v, Comp3<float> v_lo) {
+                        const double* v0, int c, float* v, float* v_lo, double* v64) {
   cx.before(-1);
-  k_velocity_dw<<<grid3(P.nx, P.ny, P.nz, 1), block3(), 0, cx.stream>>>(P, psi, psi_lo, v0d, v,
-                                                                        v_lo);
+  if (v64) velocity_dw_c<kVelF64>(cx, P, psi, psi_lo, v0, c, nullptr, nullptr, v64);
+  else if (v_lo) velocity_dw_c<kVelWords>(cx, P, psi, psi_lo, v0, c, v, v_lo, nullptr);
+  else velocity_dw_c<kVelF32>(cx, P, psi, psi_lo, v0, c, v, nullptr, nullptr);
   cx.after(-1);
 }
 
@@ -1391,21 +1622,44 @@ template <class T>
 void launch_diag(Ctx& cx, const PhaseParams& P, const T* phi, const T* phi_lo, const T* g,
                  const T* g_lo, Comp3<T> vel, Comp3<T> vel_lo, Comp3<T> omega, Comp3<T> om_lo,
                  Comp3<T> psi, Comp3<T> ps_lo, Comp3<const double> psi0_ring,
-                 Comp3<const double> v0d, T* sigma_t, double* partials, int nblocks, double* out) {
+                 Comp3<const double> v0d, double* partials, int nblocks, double* out) {
   cx.before(-1);
-  k_diag<T><<<nblocks, kBlock, 0, cx.stream>>>(P, phi, phi_lo, g, g_lo, vel, vel_lo, omega, om_lo,
-                                               psi, ps_lo, psi0_ring, v0d, sigma_t, partials);
+  k_diag_flow<T><<<nblocks, kBlock, 0, cx.stream>>>(P, vel, vel_lo, v0d, partials);
   cx.after(-1);
   cx.before(-1);
-  k_diag_finalize<<<1, kBlock, 0, cx.stream>>>(partials, nblocks, out);
+  k_diag_state<T><<<nblocks, kBlock, 0, cx.stream>>>(P, phi, phi_lo, g, g_lo, omega, om_lo, psi, ps_lo,
+                                                     psi0_ring, partials);
+  cx.after(-1);
+  cx.before(-1);
+  k_diag_finalize<<<13, kBlock, 0, cx.stream>>>(partials, nblocks, out);
   cx.after(-1);
 }
 
 template <class T>
-void launch_stress_profile(Ctx& cx, const PhaseParams& P, Comp3<T> vel, Comp3<T> vel_lo,
-                           double* out) {
+void launch_sigma_t(Ctx& cx, const PhaseParams& P, Comp3<T> vel, Comp3<T> vel_lo, T* out) {
+  const dim3 grid = grid3(P.nx, P.ny, P.nz, 1);
   cx.before(-1);
-  k_stress_profile<T><<<P.ny, kBlock, 0, cx.stream>>>(P, vel, vel_lo, out);
+  if constexpr (std::is_same<T, float>::value) {
+    const double f = 0.5 * P.inv_h / P.inv_eta, f2 = f * f;
+    const FF s{(float)f2, (float)(f2 - (double)(float)f2)};
+    k_sigma_t_dw<<<grid, block3(), 0, cx.stream>>>(P, vel, vel_lo, s, out);
+  } else {
+    k_sigma_t<<<grid, block3(), 0, cx.stream>>>(P, vel, out);
+  }
+  cx.after(-1);
+}
+
+template <class T>
+void launch_stress_profile(Ctx& cx, const PhaseParams& P, const T* vx, const T* vx_lo, double* sums,
+                           double* out) {
+  // chunks of planes so that the rows fill the SMs; sums holds ny nz doubles
+  const int chunks = std::max(1, std::min(P.nz, 4 * cx.sms / std::max(1, P.ny)));
+  const int kchunk = (P.nz + chunks - 1) / chunks, n = (P.nz + kchunk - 1) / kchunk;
+  cx.before(-1);
+  k_row_sums<T><<<dim3(P.ny, n), kBlock, 0, cx.stream>>>(P, vx, vx_lo, kchunk, sums);
+  cx.after(-1);
+  cx.before(-1);
+  k_stress_profile<<<(P.ny + 127) / 128, 128, 0, cx.stream>>>(P, sums, n, out);
   cx.after(-1);
 }
 
@@ -1486,13 +1740,13 @@ void launch_fill(Ctx& cx, double* x, long long n, double v) {
   template void launch_mu<T>(Ctx&, const PhaseParams&, const T*, T*, T*, const Scalars*);         \
   template void launch_source<T>(Ctx&, const PhaseParams&, const T*, const T*, Comp3<T>,          \
                                  Comp3<T>);                                                       \
-  template void launch_velocity<T>(Ctx&, const PhaseParams&, Comp3<T>, Comp3<T>, Comp3<T>,       \
-                                   Comp3<T>);                                                     \
+  template void launch_velocity<T>(Ctx&, const PhaseParams&, Comp3<T>, const T*, int, T*);        \
   template void launch_diag<T>(Ctx&, const PhaseParams&, const T*, const T*, const T*, const T*,  \
                                Comp3<T>, Comp3<T>, Comp3<T>, Comp3<T>, Comp3<T>, Comp3<T>,        \
-                               Comp3<const double>, Comp3<const double>, T*, double*, int,        \
-                               double*);                                                          \
-  template void launch_stress_profile<T>(Ctx&, const PhaseParams&, Comp3<T>, Comp3<T>, double*);  \
+                               Comp3<const double>, Comp3<const double>, double*, int, double*);  \
+  template void launch_sigma_t<T>(Ctx&, const PhaseParams&, Comp3<T>, Comp3<T>, T*);              \
+  template void launch_stress_profile<T>(Ctx&, const PhaseParams&, const T*, const T*, double*,   \
+                                         double*);                                                \
   template void launch_full_field<T>(Ctx&, const PhaseParams&, const T*, const T*, const double*,  \
                                      int, T*);                                                    \
   template void launch_scale_copy<T>(Ctx&, const T*, T*, long long, double);

@@ -477,9 +477,9 @@ bool smooth(vsv_grid* g, const Level& L, int l, Comp3<T> X, Rhs3<T> R, int ncomp
       return fuse_upd;
     }
   }
-  if (x_zero) launch_zero<T>(g->cx, X, L.cells(), ncomp);
+  if (x_zero && nu == 0) launch_zero<T>(g->cx, X, L.cells(), ncomp);
   for (int s = 0; s < nu; ++s) {
-    launch_rb_sweep<T>(g->cx, L, X, R, ncomp, 0, w, h2, kc);
+    launch_rb_sweep<T>(g->cx, L, X, R, ncomp, 0, w, h2, kc, x_zero && s == 0);
     launch_rb_sweep<T>(g->cx, L, X, R, ncomp, 1, w, h2, kc);
   }
   return false;
@@ -636,13 +636,10 @@ bool vcycle(vsv_grid* g, const std::vector<Level>& lv, int l, Comp3<T> X, Rhs3<T
       if (launch_coarse_solve<T>(g->cx, L, E, RR, ncomp, coarsest_sweeps(L, g->sol.coarse_sweeps),
                                  h2))
         return false;
-      launch_zero<T>(g->cx, E, L.cells(), ncomp);
-    } else if (x_zero) {
-      launch_zero<T>(g->cx, X, L.cells(), ncomp);
     }
     const int cs = coarsest_sweeps(L, g->sol.coarse_sweeps);
     for (int s = 0; s < cs; ++s) {
-      launch_rb_sweep<T>(g->cx, L, X, R, ncomp, 0, 1.0, h2, kc);
+      launch_rb_sweep<T>(g->cx, L, X, R, ncomp, 0, 1.0, h2, kc, s == 0 && (l > 0 || x_zero));
       launch_rb_sweep<T>(g->cx, L, X, R, ncomp, 1, 1.0, h2, kc);
     }
     return false;

@@ -99,11 +99,13 @@ __device__ __forceinline__ T prolong_pair(T c, T x) {   // 3/4 c + 1/4 x
   return fma_t((T)0.75, c, mul_t((T)0.25, x));
 }
 template <class T>
+__device__ __forceinline__ T prolong_sum(T a, T b, T c, T d) {   // of the four pairs
+  return fma_t((T)0.0625, d, fma_t((T)0.1875, c, fma_t((T)0.1875, b, mul_t((T)0.5625, a))));
+}
+template <class T>
 __device__ __forceinline__ T prolong_value(T aC, T aX, T bC, T bX, T cC, T cX, T dC, T dX) {
-  T acc = mul_t((T)0.5625, prolong_pair(aC, aX));
-  acc = fma_t((T)0.1875, prolong_pair(bC, bX), acc);
-  acc = fma_t((T)0.1875, prolong_pair(cC, cX), acc);
-  return fma_t((T)0.0625, prolong_pair(dC, dX), acc);
+  return prolong_sum(prolong_pair(aC, aX), prolong_pair(bC, bX), prolong_pair(cC, cX),
+                     prolong_pair(dC, dX));
 }
 
 // b - L x of one cell: (neighbour sum s) - coef x, times 1 / h^2, from b;
@@ -160,7 +162,7 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Right-hand side b = beta * B[c] + S[j + k * ny] (S may be null).
+// Right-hand side b = beta * B[c] + S[j + k * ny] (beta 1 or -1; S may be null).
 template <class T>
 struct Rhs3 {
   const T* B[3];
@@ -202,7 +204,7 @@ inline dim3 block3() { return dim3(kBX, kBY, 1); }
 __device__ __forceinline__ bool cell3(int nx, int ny, int nz, int& i, int& j, int& k, int& comp) {
   i = blockIdx.x * blockDim.x + threadIdx.x;
   j = blockIdx.y * blockDim.y + threadIdx.y;
-  comp = (int)(blockIdx.z / (unsigned)nz);
+  comp = ((int)blockIdx.z >= nz) + ((int)blockIdx.z >= 2 * nz);   // at most three components
   k = (int)blockIdx.z - comp * nz;
   return i < nx && j < ny;
 }

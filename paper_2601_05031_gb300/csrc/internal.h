@@ -133,9 +133,10 @@ __device__ __forceinline__ double block_max(double v) {
 }
 
 // ---------------------------------------------------------------- Poisson launchers (mg.cu)
+// zero (colour 0): x is taken as zero, and its other colour set to zero
 template <class T>
 void launch_rb_sweep(Ctx& cx, const Level& L, Comp3<T> X, Rhs3<T> R, int ncomp, int color,
-                     double omega, double h2, int kclass);
+                     double omega, double h2, int kclass, bool zero = false);
 template <class T>
 void launch_resid_restrict(Ctx& cx, const Level& F, const Level& C, Comp3<T> X, Rhs3<T> R,
                            Comp3<T> RC, int ncomp, bool exact);

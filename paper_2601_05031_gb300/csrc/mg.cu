@@ -64,9 +64,17 @@ __device__ __forceinline__ T sum_nb(const T* __restrict__ x, const Level& L, int
   return (s[0] + s[1]) + s[2];
 }
 
+// b with the sign of a rhs factor (1 or -1), by an integer operation, which
+// takes no FP64 unit's time.
+__device__ __forceinline__ double sign_of(double b, double beta) {
+  return __hiloint2double(__double2hiint(b) ^ (__double2hiint(beta) & (int)0x80000000u),
+                          __double2loint(b));
+}
+__device__ __forceinline__ float sign_of(float b, float beta) { return beta * b; }
+
 template <class T>
 __device__ __forceinline__ T rhs_at(const Rhs3<T>& R, int comp, long long c, int j, int k, int ny) {
-  T b = R.beta * R.b_at(comp)[c];
+  T b = sign_of(R.b_at(comp)[c], R.beta);
   if (R.s_at(comp)) b += R.s_at(comp)[j + (long long)k * ny];
   return b;
 }
@@ -120,24 +128,68 @@ __device__ __forceinline__ T resid_at(const T* __restrict__ x, const Level& L, i
 }
 
 // ---------------------------------------------------------------- sweeps
+// What a sweep kernel reads of its level, with the constants of relax()
+// rounded on the host: a launch carries a third of a Level, and a cell on the
+// FP64 path, whose units do two operations per clock and SM, spends no
+// operation on them.
+template <class T>
+struct SweepGeom {
+  int nx, ny, nz;
+  int act[3], per[3];
+  T w[7];          // omega / diagonal for 0 .. 6 wall neighbours
+  T h2, c1, beta;  // h^2 (with the sign of the rhs if it has no plane term),
+                   // 1 - omega, the sign of the rhs
+};
+
 // One colour of a red-black Gauss-Seidel sweep (omega = 1) or SOR sweep
 // (the red-black SOR solver, or over-relaxed multigrid smoothing),
 // colour = (i + j + k) & 1, in place.  Thread t handles the t-th cell of the
-// colour in its x row.
-template <class T>
-__global__ void k_rb_sweep(Level L, Comp3<T> X, Rhs3<T> R, int color, T omega, T h2) {
+// colour in its x row.  ZERO (colour 0): x is to be taken as zero and holds
+// anything: the red cells take the scaled rhs, the black ones zero, as a fill
+// and a red half-sweep leave them.
+//
+// PLANE: the rhs has a plane term (without one the sign of the rhs is in h^2).
+// A condition on it, or a factor, inside the kernel becomes a predicate, and an FP64 operation that is predicated off takes the units' time
+// like any other.  FP64: 8 operations per cell and colour (3 with ZERO) instead
+// of 12, 9 with s; 139 -> 98 us a colour at 256 x 128 x 128, three components,
+// 139 -> 110 us with s.
+template <class T, bool ZERO, bool PLANE>
+__global__ void k_rb_sweep(const __grid_constant__ SweepGeom<T> G, Comp3<T> X, Rhs3<T> R, int color) {
   pdl_begin();
-  const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
+  const int nx = G.nx, ny = G.ny, nz = G.nz;
   int i2, j, k, comp;
   if (!cell3((nx + 1) >> 1, ny, nz, i2, j, k, comp)) return;
   T* __restrict__ x = X.at(comp);
   const int i = 2 * i2 + ((j + k + color) & 1);
-  if (i >= nx) return;
   const long long c = lin(i, j, k, nx, ny);
-  int nwall;
-  const T s = sum_nb(x, L, i, j, k, c, nwall);
-  const T b = rhs_at(R, comp, c, j, k, ny);
-  x[c] = relax(x[c], nb_term(s, b, h2), wscale(omega, lv_rc<T>(L, nwall)), (T)1 - omega);
+  if (ZERO && (i ^ 1) < nx) x[c + ((i & 1) ? -1 : 1)] = (T)0;
+  if (i >= nx) return;
+  const long long sy = nx, sz = (long long)nx * ny;
+  int nwall = 0;
+  T a = 0, b = 0, s[3];
+  auto add = [&](int q, bool in, long long d, long long wrap) -> T {
+    if (!G.act[q]) return (T)0;
+    if (in) return ZERO ? (T)0 : x[c + d];
+    if (G.per[q]) return ZERO ? (T)0 : x[c + wrap];
+    ++nwall;
+    return (T)0;
+  };
+  a = add(0, i > 0, -1, nx - 1);
+  b = add(0, i < nx - 1, 1, 1 - nx);
+  s[0] = a + b;
+  a = add(1, j > 0, -sy, (ny - 1) * sy);
+  b = add(1, j < ny - 1, sy, (1 - ny) * sy);
+  s[1] = a + b;
+  a = add(2, k > 0, -sz, (nz - 1) * sz);
+  b = add(2, k < nz - 1, sz, (1 - nz) * sz);
+  s[2] = a + b;
+  const T sn = ZERO ? (T)0 : (s[0] + s[1]) + s[2];
+  T r = R.b_at(comp)[c];
+  if (PLANE) {
+    r = sign_of(r, G.beta);
+    if (R.s_at(comp)) r += R.s_at(comp)[j + (long long)k * ny];
+  }
+  x[c] = relax(ZERO ? (T)0 : x[c], nb_term(sn, r, G.h2), G.w[nwall], G.c1);
 }
 
 // Residual of the fine (or any) level, restricted to the next coarser level
@@ -394,10 +446,22 @@ __global__ void k_restrict_block(Level F, Level C, Comp3<T> X, Rhs3<T> R, Comp3<
       fxp[kz][jy] = xp >= 0 ? r[xp] : (T)0;
       const long long t = ((long long)(k0 + kz) * ny + j0 + jy) * nx + i0;
       ld2(R.b_at(comp) + t, b[kz][jy][0], b[kz][jy][1]);
-      const T s = R.s_at(comp) ? R.s_at(comp)[j0 + jy + (long long)(k0 + kz) * ny] : (T)0;
-      b[kz][jy][0] = R.beta * b[kz][jy][0] + s;
-      b[kz][jy][1] = R.beta * b[kz][jy][1] + s;
+      b[kz][jy][0] = sign_of(b[kz][jy][0], R.beta);
+      b[kz][jy][1] = sign_of(b[kz][jy][1], R.beta);
     }
+  // one branch for the plane term (per cell it becomes a predicated FP64
+  // operation, which takes the units' time all the same).  FP64: 227 -> 211 us
+  // with the sign change off the units, 256 x 128 x 128, three components
+  if (R.s_at(comp)) {
+#pragma unroll
+    for (int kz = 0; kz < 2; ++kz)
+#pragma unroll
+      for (int jy = 0; jy < 2; ++jy) {
+        const T s = R.s_at(comp)[j0 + jy + (long long)(k0 + kz) * ny];
+        b[kz][jy][0] += s;
+        b[kz][jy][1] += s;
+      }
+  }
 #pragma unroll
   for (int kz = 0; kz < 2; ++kz) {
     if (ym >= 0) ld2(row(ym, k0 + kz) + i0, fym[kz][0], fym[kz][1]); else fym[kz][0] = fym[kz][1] = (T)0;
@@ -454,26 +518,50 @@ __device__ __forceinline__ void prolong_children(const Level& C, const T* __rest
     t = outer_idx(K + d, cz, C.per[2]);
     iz[s] = t >= 0 ? t : K; fz[s] = t >= 0 ? (T)1 : ma;
   }
+  bool wall = (I == 0 || I == cx_ - 1) && !C.per[0];
+  wall = wall || ((J == 0 || J == cy - 1) && !C.per[1]);
+  wall = wall || ((K == 0 || K == cz - 1) && !C.per[2]);
   T n[3][3][3];
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const T* r = e + ((long long)iz[c] * cy + iy[b]) * cx_;
-      const T f = fz[c] * fy[b];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) n[c][b][a] = f * fx[a] * r[ix[a]];
+      for (int a = 0; a < 3; ++a) n[c][b][a] = r[ix[a]];
+    }
+  // the boundary factors are all 1 away from walls: one branch around their
+  // multiplications (per-value conditions become selects, and the FP64 units
+  // then do every product), decided on integers (an FP64 compare is an FP64
+  // operation too)
+  if (wall) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const T f = fz[c] * fy[b];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) n[c][b][a] = f * fx[a] * n[c][b][a];
+      }
+  }
+  // the x-interpolated value of each of the nine rows on the even and the odd
+  // child's side.  FP64: 76 operations per coarse cell with the eight updates
+  // instead of 167; 344 -> 209 us at 256 x 128 x 128, three components
+  T p[3][3][2];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      p[c][b][0] = prolong_pair(n[c][b][1], n[c][b][0]);
+      p[c][b][1] = prolong_pair(n[c][b][1], n[c][b][2]);
     }
 #pragma unroll
   for (int c = 0; c < 2; ++c)
 #pragma unroll
     for (int b = 0; b < 2; ++b)
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const int ax = 2 * a, by = 2 * b, cz2 = 2 * c;
-        v[c][b][a] = prolong_value<T>(n[1][1][1], n[1][1][ax], n[1][by][1], n[1][by][ax],
-                                      n[cz2][1][1], n[cz2][1][ax], n[cz2][by][1], n[cz2][by][ax]);
-      }
+      for (int a = 0; a < 2; ++a)
+        v[c][b][a] = prolong_sum(p[1][1][a], p[1][2 * b][a], p[2 * c][1][a], p[2 * c][2 * b][a]);
 }
 
 // x_fine += P e for the 8 children of one coarse cell per thread.
@@ -1425,14 +1513,36 @@ bool launch_barrier_probe(cudaStream_t s, GridBarrier B, int blocks, int rounds)
 static inline unsigned blocks_for(long long n) { return (unsigned)((n + kBlock - 1) / kBlock); }
 
 template <class T>
+static SweepGeom<T> sweep_geom(const Level& L, const Rhs3<T>& R, double omega, double h2) {
+  SweepGeom<T> G;
+  G.nx = L.n[0]; G.ny = L.n[1]; G.nz = L.n[2];
+  for (int a = 0; a < 3; ++a) {
+    G.act[a] = L.act[a];
+    G.per[a] = L.per[a];
+  }
+  const T om = (T)omega;
+  for (int q = 0; q < 7; ++q) G.w[q] = om * lv_rc<T>(L, q);
+  G.h2 = (T)h2;
+  G.c1 = (T)1 - om;
+  G.beta = R.beta;
+  return G;
+}
+
+template <class T>
 void launch_rb_sweep(Ctx& cx, const Level& L, Comp3<T> X, Rhs3<T> R, int ncomp, int color,
-                     double omega, double h2, int kclass) {
+                     double omega, double h2, int kclass, bool zero) {
   const dim3 grid = grid3((L.n[0] + 1) / 2, L.n[1], L.n[2], ncomp);
+  SweepGeom<T> G = sweep_geom<T>(L, R, omega, h2);
+  bool plane = false;
+  for (int q = 0; q < ncomp; ++q) plane = plane || R.S[q];
+  if (!plane) G.h2 *= R.beta;
+  auto kern = plane ? (zero ? k_rb_sweep<T, true, true> : k_rb_sweep<T, false, true>)
+                    : (zero ? k_rb_sweep<T, true, false> : k_rb_sweep<T, false, false>);
   cx.before(kclass);
-  launch_k(cx, k_rb_sweep<T>, grid, block3(), 0, L, X, R, color, (T)omega, (T)h2);
+  launch_k(cx, kern, grid, block3(), 0, G, X, R, color);
   // one colour: the other colour's values and this colour's rhs read, this colour written
-  // (and read, for SOR): 1.5 words per cell
-  cx.after(kclass, (omega == 1.0 ? 1.5 : 2.0) * (double)sizeof(T) * (double)L.cells() * ncomp);
+  // (and read, for SOR): 1.5 words per cell; from zero this colour's rhs read, both written
+  cx.after(kclass, (zero || omega == 1.0 ? 1.5 : 2.0) * (double)sizeof(T) * (double)L.cells() * ncomp);
 }
 
 template <class T>
@@ -1549,7 +1659,7 @@ void launch_norm_finalize(Ctx& cx, const double* partials, int nblocks, int ncom
 
 #define VSV_INST(T)                                                                                \
   template void launch_rb_sweep<T>(Ctx&, const Level&, Comp3<T>, Rhs3<T>, int, int, double, double, \
-                                   int);                                                           \
+                                   int, bool);                                                     \
   template void launch_resid_restrict<T>(Ctx&, const Level&, const Level&, Comp3<T>, Rhs3<T>,      \
                                          Comp3<T>, int, bool);                                     \
   template void launch_prolong_add<T>(Ctx&, const Level&, const Level&, Comp3<T>, Comp3<T>, int);  \

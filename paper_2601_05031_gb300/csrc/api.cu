@@ -109,6 +109,10 @@ struct vsv_grid {
   double omega_dt = 0.0;
   int* flag_host = nullptr;        // pinned copy of the device non-finite flag
   int* flag_dev = nullptr;         // its device address (mapped)
+  // the three components' (||r||^2, ||b||^2) of a residual check, in the same
+  // page-locked allocation, and their device address
+  double* norm_host = nullptr;
+  double* norm_dev = nullptr;
   // component-parallel flow solves: the first component of the
   // per-component scratch the current solve uses, the two extra streams the
   // components 1 and 2 run on, and the events that fork and join them
@@ -692,13 +696,12 @@ bool vcycle(vsv_grid* g, const std::vector<Level>& lv, int l, Comp3<T> X, Rhs3<T
 template <class T>
 vsv_status residual(vsv_grid* g, const Level& L, Comp3<T> X, Rhs3<T> R, int ncomp, double* relres) {
   launch_resid_norm<T>(g->cx, L, X, R, ncomp, std::is_same<T, float>::value, g->partials,
-                       g->red_blocks, g->S);
-  Scalars hs;
-  CK(cudaMemcpyAsync(&hs, g->S, sizeof(Scalars), cudaMemcpyDeviceToHost, g->cx.stream));
+                       g->red_blocks, g->S, g->norm_dev);
   CK(cudaStreamSynchronize(g->cx.stream));
+  CKL();
   double m = 0.0;
   for (int c = 0; c < ncomp; ++c) {
-    const double rn = std::sqrt(hs.rnorm2[c]), bn = std::sqrt(hs.bnorm2[c]);
+    const double rn = std::sqrt(g->norm_host[2 * c]), bn = std::sqrt(g->norm_host[2 * c + 1]);
     m = std::max(m, bn > 0 ? rn / bn : rn);
   }
   *relres = m;
@@ -780,17 +783,17 @@ vsv_status solve_dc(vsv_grid* g, const std::vector<Level>& lv, Comp3<float> XH, 
     if (!vcycle<float>(g, lv, 0, E, RE, ncomp, false, true, &XH, &XL))
       launch_update_dw(g->cx, XH, XL, E, L.cells(), ncomp);
   };
-  // defect r = b - L x (tiled kernel where the level allows it); returns the
-  // number of partial-sum blocks per component written when `norms`
-  auto defect = [&](bool norms) -> int {
+  // defect r = b - L x (tiled kernel where the level allows it), with `norms`
+  // also its norms and the rhs's
+  auto defect = [&](bool norms) {
     double* part = norms ? g->partials : nullptr;
     if (g->sol.variant != 1) {
-      const int nb = launch_defect_tiled(g->cx, L, XH, XL, R, BL, RR, ncomp, part,
-                                         g->red_blocks * 32 / (2 * ncomp), g->sol.variant == 0);
-      if (nb > 0) return nb;
+      if (launch_defect_tiled(g->cx, L, XH, XL, R, BL, RR, ncomp, part,
+                              g->red_blocks * 32 / (2 * ncomp), g->sol.variant == 0, g->S,
+                              g->norm_dev) > 0)
+        return;
     }
-    launch_defect_dw(g->cx, L, XH, XL, R, BL, RR, ncomp, part, g->red_blocks);
-    return g->red_blocks;
+    launch_defect_dw(g->cx, L, XH, XL, R, BL, RR, ncomp, part, g->red_blocks, g->S, g->norm_dev);
   };
   if (fixed > 0) {
     for (int c = 0; c < fixed; ++c) {
@@ -807,15 +810,13 @@ vsv_status solve_dc(vsv_grid* g, const std::vector<Level>& lv, Comp3<float> XH, 
   double rr = INFINITY;
   while (true) {
     const bool check = (c % every == 0) || c >= max_cycles;
-    const int nb = defect(check);
+    defect(check);
     if (check) {
-      launch_norm_finalize(g->cx, g->partials, nb, ncomp, g->S);
-      Scalars hs;
-      CK(cudaMemcpyAsync(&hs, g->S, sizeof(Scalars), cudaMemcpyDeviceToHost, g->cx.stream));
       CK(cudaStreamSynchronize(g->cx.stream));
+      CKL();
       rr = 0.0;
       for (int q = 0; q < ncomp; ++q) {
-        const double rn = std::sqrt(hs.rnorm2[q]), bn = std::sqrt(hs.bnorm2[q]);
+        const double rn = std::sqrt(g->norm_host[2 * q]), bn = std::sqrt(g->norm_host[2 * q + 1]);
         rr = std::max(rr, bn > 0 ? rn / bn : rn);
       }
       if (rr <= tol || c >= max_cycles) break;
@@ -1626,7 +1627,7 @@ vsv_status vsv_create(vsv_grid** out, int nx, int ny, int nz, double h, int prec
   }
   // the handle's page-locked word for vsv_step's deferred status, and the
   // event that marks its arrival (created here: stepping allocates nothing)
-  bool ok = cudaMallocHost((void**)&g->flag_host, sizeof(int)) == cudaSuccess &&
+  bool ok = cudaMallocHost((void**)&g->flag_host, 64 + 6 * sizeof(double)) == cudaSuccess &&
             cudaHostGetDevicePointer((void**)&g->flag_dev, g->flag_host, 0) == cudaSuccess &&
             cudaEventCreateWithFlags(&g->flag_event, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&g->fork_ev, cudaEventDisableTiming) == cudaSuccess &&
@@ -1644,6 +1645,8 @@ vsv_status vsv_create(vsv_grid** out, int nx, int ny, int nz, double h, int prec
     return VSV_ECUDA;
   }
   *g->flag_host = 0;
+  g->norm_host = (double*)((char*)g->flag_host + 64);
+  g->norm_dev = (double*)((char*)g->flag_dev + 64);
   upload_scalar_params(g);
   *out = g;
   return VSV_OK;

@@ -182,10 +182,9 @@ struct Scalars {
   double lambda_v, gamma_a;
   double k_vol, k_area, eps;   // copies of the penalty parameters
   double h3;
-  double rnorm2[3], bnorm2[3];
   float lambda_vf, gamma_af;   // FP32 copies read by the FP32 kernels
   int nonfinite;
-  int pad;
+  unsigned ticket;             // CTAs of a norm reduction that have stored their sums
 };
 
 // ---------------------------------------------------------------- device helpers

@@ -54,7 +54,7 @@ __device__ __forceinline__ float defect_combine(float b1, float b2, bool has_b2,
 // block.
 __global__ void k_defect_dw(Level L, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R,
                             Comp3<float> BL, Comp3<float> OUT, double* partials, float ih_hi,
-                            float ih_lo) {
+                            float ih_lo, Scalars* SC, double* host) {
   pdl_begin();
   const int comp = blockIdx.y;
   const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
@@ -68,11 +68,13 @@ __global__ void k_defect_dw(Level L, Comp3<float> XH, Comp3<float> XL, Rhs3<floa
   // diagonal 2 d + s h^2 as a pair (alpha = 0 on the finest level)
   const float dch = L.cdh[0], dcl = L.cdl[0];
   double rr = 0.0, bb = 0.0;
-  for (int row = blockIdx.x; row < ny * nz; row += gridDim.x) {
-    const int j = row % ny, k = row / ny;
+  const int lanes = row_lanes(nx);
+  for (int row = (blockIdx.x * kBlock + threadIdx.x) / lanes; row < ny * nz;
+       row += gridDim.x * kBlock / lanes) {
+    const int k = row / ny, j = row - k * ny;
     const float s = S ? S[j + (long long)k * ny] : 0.f;
     float r2 = 0.f, b2 = 0.f;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+    for (int i = threadIdx.x & (lanes - 1); i < nx; i += lanes) {
       const long long t = lin(i, j, k, nx, ny);
       // hi words: cascade from the first active direction's x- neighbour
       // on, in the order x-, x+, y-, y+, z-, z+; lo words: the per-axis
@@ -110,13 +112,8 @@ __global__ void k_defect_dw(Level L, Comp3<float> XH, Comp3<float> XL, Rhs3<floa
     bb += (double)b2;
   }
   if (partials) {
-    rr = block_sum(rr);
-    bb = block_sum(bb);
-    if (threadIdx.x == 0) {
-      double* o = partials + ((long long)comp * gridDim.x + blockIdx.x) * 2;
-      o[0] = rr;
-      o[1] = bb;
-    }
+    __shared__ double buf[2 * kBlock];
+    norm_publish(rr, bb, buf, partials, gridDim.x, gridDim.y, comp, blockIdx.x, SC, host);
   }
 }
 
@@ -184,11 +181,12 @@ __global__ void k_axpy_dw(Comp3<float> YH, Comp3<float> YL, Comp3<float> XH, Com
 }
 
 void launch_defect_dw(Ctx& cx, const Level& L, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R,
-                      Comp3<float> BL, Comp3<float> OUT, int ncomp, double* partials, int nblocks) {
+                      Comp3<float> BL, Comp3<float> OUT, int ncomp, double* partials, int nblocks,
+                      Scalars* S, double* host) {
   const float ih_hi = (float)L.inv_h2, ih_lo = (float)(L.inv_h2 - (double)ih_hi);
-  dim3 grid(nblocks, ncomp);
+  dim3 grid(row_blocks(L, nblocks), ncomp);
   cx.before(VSV_KCLASS_RESTRICT);
-  launch_k(cx, k_defect_dw, grid, kBlock, 0, L, XH, XL, R, BL, OUT, partials, ih_hi, ih_lo);
+  launch_k(cx, k_defect_dw, grid, kBlock, 0, L, XH, XL, R, BL, OUT, partials, ih_hi, ih_lo, S, host);
   cx.after(VSV_KCLASS_RESTRICT, (BL.p[0] ? 20.0 : 16.0) * (double)L.cells() * ncomp);
 }
 
@@ -250,7 +248,7 @@ __device__ __forceinline__ float defect_cell(float xmh, float xph, float ymh, fl
 template <int ROWS, bool RAGGED, bool NORMS>
 __global__ void __launch_bounds__(tile::kThreads, ROWS == 1 ? 3 : 2)
 k_defect_tiled(DefGeom G, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R, Comp3<float> BL,
-               Comp3<float> OUT, double* partials) {
+               Comp3<float> OUT, double* partials, Scalars* SC, double* host) {
   pdl_begin();
   using namespace tile;
   constexpr int kDR = DefShape<ROWS>::kDR, kRows = DefShape<ROWS>::kRows;
@@ -385,14 +383,9 @@ k_defect_tiled(DefGeom G, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R, Comp3
   }
   cp_async_wait0();
   if (NORMS) {
-    rr = block_sum(rr);
-    bb = block_sum(bb);
-    if (threadIdx.x == 0) {
-      const long long nb = (long long)gridDim.x * gridDim.y;
-      double* o = partials + ((long long)comp * nb + blockIdx.x + (long long)gridDim.x * blockIdx.y) * 2;
-      o[0] = rr;
-      o[1] = bb;
-    }
+    static_assert(kThreads == kBlock && DefShape<ROWS>::kSmem >= 2 * kBlock * sizeof(double), "");
+    norm_publish(rr, bb, reinterpret_cast<double*>(smem_d4), partials, gridDim.x * gridDim.y, gridDim.z, comp,
+                 blockIdx.x + gridDim.x * blockIdx.y, SC, host);
   }
 }
 
@@ -400,7 +393,7 @@ k_defect_tiled(DefGeom G, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R, Comp3
 // partial-sum blocks per component (0 if it did not launch)
 int launch_defect_tiled(Ctx& cx, const Level& L, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R,
                         Comp3<float> BL, Comp3<float> OUT, int ncomp, double* partials, int max_blocks,
-                        bool ragged) {
+                        bool ragged, Scalars* S, double* host) {
   const bool aligned = tile::level_ok(L);
   if (!aligned && !(ragged && tile::ragged_ok(L) && tile::tile_fill(L) >= 0.25 &&
                     L.cells() >= (1 << 17)))
@@ -442,7 +435,7 @@ int launch_defect_tiled(Ctx& cx, const Level& L, Comp3<float> XH, Comp3<float> X
   auto kern = aligned ? (partials ? k_defect_tiled<ROWS, false, true> : k_defect_tiled<ROWS, false, false>)
                       : (partials ? k_defect_tiled<ROWS, true, true> : k_defect_tiled<ROWS, true, false>);
   cx.before(VSV_KCLASS_RESTRICT);
-  launch_k(cx, kern, grid, tile::kThreads, Sh::kSmem, G, XH, XL, R, BL, OUT, partials);
+  launch_k(cx, kern, grid, tile::kThreads, Sh::kSmem, G, XH, XL, R, BL, OUT, partials, S, host);
   // x_hi, x_lo, b_hi (, b_lo) read, r written
   cx.after(VSV_KCLASS_RESTRICT, (BL.p[0] ? 20.0 : 16.0) * (double)L.cells() * ncomp);
   return tiles * nz;

@@ -132,6 +132,74 @@ __device__ __forceinline__ double block_max(double v) {
   return r;
 }
 
+// Threads of a CTA of kBlock that share a row of nx cells in the row-wise
+// reductions: the least power of two from 32 on that covers it, so that short
+// rows leave no warp idle and a thread still adds one cell of a row (of up to
+// 256) before its sum goes to FP64; and the CTAs per component that one pass
+// over the rows then takes, at most max_blocks.
+__host__ __device__ inline int row_lanes(int nx) {
+  return nx > 128 ? 256 : (nx > 64 ? 128 : (nx > 32 ? 64 : 32));
+}
+static_assert(kBlock == 256, "row_lanes covers a CTA's threads");
+inline unsigned row_blocks(const Level& L, int max_blocks) {
+  const long long per = kBlock / row_lanes(L.n[0]), rows = (long long)L.n[1] * L.n[2];
+  const long long b = (rows + per - 1) / per;
+  return (unsigned)(b < max_blocks ? b : max_blocks);
+}
+
+// Totals of a norm reduction: every CTA (kBlock threads) of a grid of nblocks x
+// ncomp calls this with its threads' (rr, bb) sums and a shared buffer of 2
+// kBlock doubles (which may still be read by other warps on entry); the last
+// CTA to arrive adds the partial sums of every component in a fixed order and
+// writes ||r||^2 and ||b||^2 to page-locked host memory (three pairs), so that a
+// residual check is one kernel and one synchronisation, where it was two
+// kernels, a copy into pageable memory and the same synchronisation.  A sum is
+// one warp's work (12 warp-wide FP64 additions for a CTA's threads; shuffles in
+// every warp take 45, at 16 clocks of the SM's FP64 units each).  The ticket
+// wraps to zero.  FP64 residual at 48 x 24 x 24, three components: 17.4 + 3.8 ->
+// 13.0 us; mixed defect at 64 x 32 x 32: 16.7 + 4.3 -> 10.2 us.
+__device__ __forceinline__ void norm_publish(double rr, double bb, double* buf, double* partials,
+                                             int nblocks, int ncomp, int comp, int block, Scalars* S,
+                                             double* host) {
+  __shared__ int last;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();
+  buf[threadIdx.x] = rr;
+  buf[kBlock + threadIdx.x] = bb;
+  __syncthreads();
+  if (w < 2) {
+    double v = 0.0;
+#pragma unroll
+    for (int i = 0; i < kBlock; i += 32) v += buf[w * kBlock + i + lane];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) {
+      partials[((long long)comp * nblocks + block) * 2 + w] = v;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned n = (unsigned)(nblocks * ncomp);
+    last = atomicInc(&S->ticket, n - 1) == n - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last || w >= 2 * ncomp) return;
+  const double* p = partials + (long long)(w >> 1) * nblocks * 2 + (w & 1);
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  int i = lane;
+  for (; i + 96 < nblocks; i += 128)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] += __ldcg(p + 2LL * (i + 32 * q));
+  for (; i < nblocks; i += 32) v[0] += __ldcg(p + 2LL * i);
+  v[0] = (v[0] + v[1]) + (v[2] + v[3]);
+  for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  if (lane == 0) {
+    *reinterpret_cast<volatile double*>(host + w) = v[0];
+    __threadfence_system();
+  }
+}
+
 // ---------------------------------------------------------------- Poisson launchers (mg.cu)
 // zero (colour 0): x is taken as zero, and its other colour set to zero
 template <class T>
@@ -156,7 +224,7 @@ bool launch_coarse_solve(Ctx& cx, const Level& L, Comp3<T> E, Comp3<T> R, int nc
                          double h2);
 template <class T>
 void launch_resid_norm(Ctx& cx, const Level& L, Comp3<T> X, Rhs3<T> R, int ncomp, bool exact,
-                       double* partials, int nblocks, Scalars* S);
+                       double* partials, int nblocks, Scalars* S, double* host);
 
 // Lower part of a V-cycle (levels first .. last) run by one CTA per component
 // in shared memory: E (level first) <- approximate solution of L e = R.
@@ -219,18 +287,18 @@ int barrier_probe_max_blocks(int sms);
 
 // outer defect correction with double-word iterates (dc.cu)
 void launch_defect_dw(Ctx& cx, const Level& L, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R,
-                      Comp3<float> BL, Comp3<float> OUT, int ncomp, double* partials, int nblocks);
+                      Comp3<float> BL, Comp3<float> OUT, int ncomp, double* partials, int nblocks,
+                      Scalars* S, double* host);
 void launch_update_dw(Ctx& cx, Comp3<float> XH, Comp3<float> XL, Comp3<float> E, long long n,
                       int ncomp);
 // ragged: also levels that are not tile multiples (partial edge tiles)
 int launch_defect_tiled(Ctx& cx, const Level& L, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R,
                         Comp3<float> BL, Comp3<float> OUT, int ncomp, double* partials,
-                        int max_blocks, bool ragged);
+                        int max_blocks, bool ragged, Scalars* S, double* host);
 // first guess of order 0..2 from (A, B, C) = (x^n, x^{n-1}, x^{n-2}), written into C
 void launch_extrapolate_rot_dw(Ctx& cx, Comp3<float> AH, Comp3<float> AL, Comp3<float> BH,
                                Comp3<float> BL, Comp3<float> CH, Comp3<float> CL, long long n,
                                int ncomp, int order);
-void launch_norm_finalize(Ctx& cx, const double* partials, int nblocks, int ncomp, Scalars* S);
 // (YH, YL) += a (XH, XL), double-word
 void launch_axpy_dw(Ctx& cx, Comp3<float> YH, Comp3<float> YL, Comp3<float> XH, Comp3<float> XL,
                     double a, long long n, int ncomp);

@@ -149,10 +149,11 @@ struct SweepGeom {
 // and a red half-sweep leave them.
 //
 // PLANE: the rhs has a plane term (without one the sign of the rhs is in h^2).
-// A condition on it, or a factor, inside the kernel becomes a predicate, and an FP64 operation that is predicated off takes the units' time
-// like any other.  FP64: 8 operations per cell and colour (3 with ZERO) instead
-// of 12, 9 with s; 139 -> 98 us a colour at 256 x 128 x 128, three components,
-// 139 -> 110 us with s.
+// A condition on it, or a factor, inside the kernel becomes a predicate, and an
+// FP64 operation that is predicated off takes the units' time like any other.
+// FP64: 8 operations per cell and colour (3 with ZERO) instead of 12, 9 with
+// PLANE; 139 -> 98 us a colour at 256 x 128 x 128, three components, 139 -> 110
+// us with PLANE.
 template <class T, bool ZERO, bool PLANE>
 __global__ void k_rb_sweep(const __grid_constant__ SweepGeom<T> G, Comp3<T> X, Rhs3<T> R, int color) {
   pdl_begin();
@@ -348,19 +349,21 @@ __global__ void k_coarse_solve(Level L, Comp3<T> E, Comp3<T> RR, int sweeps, T h
   for (long long t = threadIdx.x; t < n; t += blockDim.x) E.at(comp)[t] = e[t];
 }
 
-// Per-block partial sums of ||b - L x||^2 and ||b||^2 (FP64 accumulation).
+// ||b - L x||^2 and ||b||^2 (FP64 accumulation), published by norm_publish, with
+// row_lanes threads on each row.
 template <class T, bool EXACT>
-__global__ void k_resid_norm(Level L, Comp3<T> X, Rhs3<T> R, double* partials, float ih_hi,
-                             float ih_lo) {
+__global__ void k_resid_norm(const __grid_constant__ Level L, Comp3<T> X, Rhs3<T> R, double* partials,
+                             float ih_hi, float ih_lo, Scalars* S, double* host) {
   pdl_begin();
   const int comp = blockIdx.y;
   const T* __restrict__ x = X.at(comp);
-  const int rows = L.n[1] * L.n[2];
+  const int rows = L.n[1] * L.n[2], lanes = row_lanes(L.n[0]);
   double rr = 0.0, bb = 0.0;
-  for (int row = blockIdx.x; row < rows; row += gridDim.x) {
-    const int j = row % L.n[1], k = row / L.n[1];
+  for (int row = (blockIdx.x * kBlock + threadIdx.x) / lanes; row < rows;
+       row += gridDim.x * kBlock / lanes) {
+    const int k = row / L.n[1], j = row - k * L.n[1];
     T r2 = 0, b2 = 0;   // per-row partial in T, then FP64 across rows
-    for (int i = threadIdx.x; i < L.n[0]; i += blockDim.x) {
+    for (int i = threadIdx.x & (lanes - 1); i < L.n[0]; i += lanes) {
       const long long t = lin(i, j, k, L.n[0], L.n[1]);
       const T b = rhs_at(R, comp, t, j, k, L.n[1]);
       const T r = resid_at<T, EXACT>(x, L, i, j, k, t, b, ih_hi, ih_lo);
@@ -370,30 +373,8 @@ __global__ void k_resid_norm(Level L, Comp3<T> X, Rhs3<T> R, double* partials, f
     rr += (double)r2;
     bb += (double)b2;
   }
-  rr = block_sum(rr);
-  bb = block_sum(bb);
-  if (threadIdx.x == 0) {
-    double* out = partials + ((long long)comp * gridDim.x + blockIdx.x) * 2;
-    out[0] = rr;
-    out[1] = bb;
-  }
-}
-
-// Sum the partials of k_resid_norm in a fixed order (one block per comp).
-__global__ void k_norm_finalize(const double* partials, int nblocks, Scalars* S) {
-  pdl_begin();
-  const int comp = blockIdx.x;
-  double rr = 0.0, bb = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-    rr += partials[((long long)comp * nblocks + b) * 2];
-    bb += partials[((long long)comp * nblocks + b) * 2 + 1];
-  }
-  rr = block_sum(rr);
-  bb = block_sum(bb);
-  if (threadIdx.x == 0) {
-    S->rnorm2[comp] = rr;
-    S->bnorm2[comp] = bb;
-  }
+  __shared__ double buf[2 * kBlock];
+  norm_publish(rr, bb, buf, partials, gridDim.x, gridDim.y, comp, blockIdx.x, S, host);
 }
 
 // ---------------------------------------------------------------- blocked transfers
@@ -1633,27 +1614,18 @@ bool launch_coarse_solve(Ctx& cx, const Level& L, Comp3<T> E, Comp3<T> R, int nc
 
 template <class T>
 void launch_resid_norm(Ctx& cx, const Level& L, Comp3<T> X, Rhs3<T> R, int ncomp, bool exact,
-                       double* partials, int nblocks, Scalars* S) {
-  dim3 grid(nblocks, ncomp);
+                       double* partials, int nblocks, Scalars* S, double* host) {
+  dim3 grid(row_blocks(L, nblocks), ncomp);
   float ih_hi = (float)L.inv_h2, ih_lo = (float)(L.inv_h2 - (double)ih_hi);
   cx.before(-1);
   if constexpr (std::is_same<T, float>::value) {
     if (exact)
-      launch_k(cx, k_resid_norm<float, true>, grid, kBlock, 0, L, X, R, partials, ih_hi, ih_lo);
+      launch_k(cx, k_resid_norm<float, true>, grid, kBlock, 0, L, X, R, partials, ih_hi, ih_lo, S, host);
     else
-      launch_k(cx, k_resid_norm<float, false>, grid, kBlock, 0, L, X, R, partials, ih_hi, ih_lo);
+      launch_k(cx, k_resid_norm<float, false>, grid, kBlock, 0, L, X, R, partials, ih_hi, ih_lo, S, host);
   } else {
-    launch_k(cx, k_resid_norm<T, false>, grid, kBlock, 0, L, X, R, partials, ih_hi, ih_lo);
+    launch_k(cx, k_resid_norm<T, false>, grid, kBlock, 0, L, X, R, partials, ih_hi, ih_lo, S, host);
   }
-  cx.after(-1);
-  cx.before(-1);
-  launch_k(cx, k_norm_finalize, ncomp, kBlock, 0, partials, nblocks, S);
-  cx.after(-1);
-}
-
-void launch_norm_finalize(Ctx& cx, const double* partials, int nblocks, int ncomp, Scalars* S) {
-  cx.before(-1);
-  launch_k(cx, k_norm_finalize, ncomp, kBlock, 0, partials, nblocks, S);
   cx.after(-1);
 }
 
@@ -1670,7 +1642,7 @@ void launch_norm_finalize(Ctx& cx, const double* partials, int nblocks, int ncom
   template bool launch_lower_vcycle<T>(Ctx&, const LowerCycle<T>&);                                \
   template bool launch_coarse_solve<T>(Ctx&, const Level&, Comp3<T>, Comp3<T>, int, int, double);  \
   template void launch_resid_norm<T>(Ctx&, const Level&, Comp3<T>, Rhs3<T>, int, bool, double*,    \
-                                     int, Scalars*);
+                                     int, Scalars*, double*);
 VSV_INST(float)
 VSV_INST(double)
 #undef VSV_INST

@@ -1269,9 +1269,9 @@ const void* mapped_host(const void* p) {
 }
 
 // Device memory of the current device with elements of `size` bytes in
-// alignment: a kernel may write a field there itself.  Anything else (another
-// device's memory, host pointers, odd offsets) gets its field by a copy.
-bool kernel_writable(const void* p, size_t size) {
+// alignment: a kernel may read or write a field there itself.  Anything else
+// (another device's memory, host pointers, odd offsets) goes by a copy.
+bool kernel_reachable(const void* p, size_t size) {
   cudaPointerAttributes a;
   int dev = -1;
   if ((uintptr_t)p % size || cudaPointerGetAttributes(&a, p) != cudaSuccess ||
@@ -1381,7 +1381,7 @@ vsv_status get_field_impl(vsv_grid* g, int field, void* dst, int dt, int on_devi
   // where a kernel writes the exported field: straight into the caller's device
   // memory, else into the staging buffer, from which deliver() copies it
   const size_t out_sz = dt == VSV_DTYPE_F64 ? 8 : 4;
-  const bool direct = on_device && kernel_writable(dst, out_sz);
+  const bool direct = on_device && kernel_reachable(dst, out_sz);
   void* const to = direct ? dst : g->stage_a;
   auto deliver = [&]() -> vsv_status {
     CKL();
@@ -2164,14 +2164,17 @@ vsv_status vsv_solve_poisson(vsv_grid* g, const void* rhs, void* x, int dtype, i
     float* xl = (float*)g->f[2];
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     auto split_in = [&](const void* src, float* hi, float* lo) -> vsv_status {
-      if (dtype == VSV_DTYPE_F64) {
+      if (dtype == VSV_DTYPE_F64 && on_device && kernel_reachable(src, 8)) {
+        launch_split_ff(g->cx, (const double*)src, hi, lo, g->N);
+      } else if (dtype == VSV_DTYPE_F64) {
         CK(cudaMemcpyAsync(g->stage_b, src, g->N * 8, kind, g->cx.stream));
         launch_split_ff(g->cx, (const double*)g->stage_b, hi, lo, g->N);
       } else {
         CK(cudaMemcpyAsync(hi, src, g->N * 4, kind, g->cx.stream));
         CK(cudaMemsetAsync(lo, 0, g->N * 4, g->cx.stream));
       }
-      CK(cudaStreamSynchronize(g->cx.stream));
+      if (!on_device) CK(cudaStreamSynchronize(g->cx.stream));
+      CKL();
       return VSV_OK;
     };
     vsv_status s = split_in(rhs, bh, bl);
@@ -2183,7 +2186,10 @@ vsv_status vsv_solve_poisson(vsv_grid* g, const void* rhs, void* x, int dtype, i
     vsv_status s2 = solve_dc(g, lv, XH, XL, R, BL, 1, 0, tol, max_cycles, g->sol.check_every,
                              cycles_out, relres_out);
     const cudaMemcpyKind okind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (dtype == VSV_DTYPE_F64) {
+    if (dtype == VSV_DTYPE_F64 && on_device && kernel_reachable(x, 8)) {
+      launch_merge_ff(g->cx, xh, xl, (double*)x, g->N);
+      CKL();
+    } else if (dtype == VSV_DTYPE_F64) {
       launch_merge_ff(g->cx, xh, xl, (double*)g->stage_b, g->N);
       CK(cudaMemcpyAsync(x, g->stage_b, g->N * 8, okind, g->cx.stream));
     } else {

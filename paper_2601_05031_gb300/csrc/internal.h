@@ -141,31 +141,29 @@ __host__ __device__ inline int row_lanes(int nx) {
   return nx > 128 ? 256 : (nx > 64 ? 128 : (nx > 32 ? 64 : 32));
 }
 static_assert(kBlock == 256, "row_lanes covers a CTA's threads");
-inline unsigned row_blocks(const Level& L, int max_blocks) {
-  const long long per = kBlock / row_lanes(L.n[0]), rows = (long long)L.n[1] * L.n[2];
-  const long long b = (rows + per - 1) / per;
+inline unsigned row_blocks(int lanes, long long rows, int max_blocks) {
+  const long long per = kBlock / lanes, b = (rows + per - 1) / per;
   return (unsigned)(b < max_blocks ? b : max_blocks);
 }
+inline unsigned row_blocks(const Level& L, int max_blocks) {
+  return row_blocks(row_lanes(L.n[0]), (long long)L.n[1] * L.n[2], max_blocks);
+}
 
-// Totals of a norm reduction: every CTA (kBlock threads) of a grid of nblocks x
-// ncomp calls this with its threads' (rr, bb) sums and a shared buffer of 2
-// kBlock doubles (which may still be read by other warps on entry); the last
-// CTA to arrive adds the partial sums of every component in a fixed order and
-// writes ||r||^2 and ||b||^2 to page-locked host memory (three pairs), so that a
-// residual check is one kernel and one synchronisation, where it was two
-// kernels, a copy into pageable memory and the same synchronisation.  A sum is
-// one warp's work (12 warp-wide FP64 additions for a CTA's threads; shuffles in
-// every warp take 45, at 16 clocks of the SM's FP64 units each).  The ticket
-// wraps to zero.  FP64 residual at 48 x 24 x 24, three components: 17.4 + 3.8 ->
-// 13.0 us; mixed defect at 64 x 32 x 32: 16.7 + 4.3 -> 10.2 us.
-__device__ __forceinline__ void norm_publish(double rr, double bb, double* buf, double* partials,
-                                             int nblocks, int ncomp, int comp, int block, Scalars* S,
-                                             double* host) {
+// Sums of two numbers over a grid of nblocks x ncomp CTAs of kBlock threads, per
+// component: every CTA calls this with its threads' (a, b) and a shared buffer
+// of 2 kBlock doubles (which may still be read by other warps on entry).  The
+// last CTA to arrive gets true, with the components' totals (a, b, a, b ..) at
+// the start of its buffer, added up from the CTAs' partial sums in a fixed
+// order: one kernel where it was two.  A sum is one warp's work: 12 warp-wide
+// FP64 additions for a CTA's threads, where shuffles in every warp take 45, at
+// 16 clocks of the SM's FP64 units each.  The ticket wraps to zero.
+__device__ __forceinline__ bool grid_sums(double a, double b, double* buf, double* partials,
+                                          int nblocks, int ncomp, int comp, int block, Scalars* S) {
   __shared__ int last;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __syncthreads();
-  buf[threadIdx.x] = rr;
-  buf[kBlock + threadIdx.x] = bb;
+  buf[threadIdx.x] = a;
+  buf[kBlock + threadIdx.x] = b;
   __syncthreads();
   if (w < 2) {
     double v = 0.0;
@@ -184,18 +182,34 @@ __device__ __forceinline__ void norm_publish(double rr, double bb, double* buf, 
     __threadfence();
   }
   __syncthreads();
-  if (!last || w >= 2 * ncomp) return;
-  const double* p = partials + (long long)(w >> 1) * nblocks * 2 + (w & 1);
-  double v[4] = {0.0, 0.0, 0.0, 0.0};
-  int i = lane;
-  for (; i + 96 < nblocks; i += 128)
+  if (!last) return false;
+  if (w < 2 * ncomp) {
+    const double* p = partials + (long long)(w >> 1) * nblocks * 2 + (w & 1);
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    int i = lane;
+    for (; i + 96 < nblocks; i += 128)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] += __ldcg(p + 2LL * (i + 32 * q));
-  for (; i < nblocks; i += 32) v[0] += __ldcg(p + 2LL * i);
-  v[0] = (v[0] + v[1]) + (v[2] + v[3]);
-  for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-  if (lane == 0) {
-    *reinterpret_cast<volatile double*>(host + w) = v[0];
+      for (int q = 0; q < 4; ++q) v[q] += __ldcg(p + 2LL * (i + 32 * q));
+    for (; i < nblocks; i += 32) v[0] += __ldcg(p + 2LL * i);
+    v[0] = (v[0] + v[1]) + (v[2] + v[3]);
+    for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    if (lane == 0) buf[w] = v[0];
+  }
+  __syncthreads();
+  return true;
+}
+
+// ||r||^2 and ||b||^2 of every component into page-locked host memory (three
+// pairs), so that a residual check is one kernel and one synchronisation, where
+// it was two kernels, a copy into pageable memory and the same synchronisation.
+// FP64 residual at 48 x 24 x 24, three components: 17.4 + 3.8 -> 13.0 us; mixed
+// defect at 64 x 32 x 32: 16.7 + 4.3 -> 10.2 us.
+__device__ __forceinline__ void norm_publish(double rr, double bb, double* buf, double* partials,
+                                             int nblocks, int ncomp, int comp, int block, Scalars* S,
+                                             double* host) {
+  if (!grid_sums(rr, bb, buf, partials, nblocks, ncomp, comp, block, S)) return;
+  if (threadIdx.x < 2 * ncomp) {
+    reinterpret_cast<volatile double*>(host)[threadIdx.x] = buf[threadIdx.x];
     __threadfence_system();
   }
 }

@@ -97,15 +97,38 @@ __global__ void k_phi_update(PhaseParams P, const T* __restrict__ phi, const T* 
 }
 
 // ---------------------------------------------------------------- reductions (SM eqs. 32, 37)
+// V, A and the penalty multipliers lambda_V = K_V (V - V0), gamma_A = K_A (A -
+// A0) 3 eps / (2 sqrt 2), by the last CTA of the reduction (15.8 + 7.2 -> 14.4 us at
+// 128 x 64 x 64 against a kernel of its own and CTAs without rows).
+__device__ __forceinline__ void va_publish(double sphi, double sarea, double* buf, double* partials,
+                                           long long ncells, Scalars* S, int init) {
+  if (!grid_sums(sphi, sarea, buf, partials, gridDim.x, 1, 0, blockIdx.x, S)) return;
+  if (threadIdx.x == 0) {
+    const double V = 0.5 * S->h3 * ((double)ncells - buf[0]);
+    const double A = S->h3 * buf[1];
+    S->V = V;
+    S->A = A;
+    if (init) {
+      S->V0 = V;
+      S->A0 = A;
+    }
+    S->lambda_v = S->k_vol * (V - S->V0);
+    S->gamma_a = S->k_area * (A - S->A0) * 3.0 * S->eps / (2.0 * 1.4142135623730951);
+    S->lambda_vf = (float)S->lambda_v;
+    S->gamma_af = (float)S->gamma_a;
+  }
+}
+
 // Per-block partial sums of sum(phi) and of the area density
 // 3/(2 sqrt2) [eps/2 |grad phi|^2 + (phi^2 - 1)^2 / (4 eps)].
 template <class T>
 __global__ void k_reduce_va(PhaseParams P, const T* __restrict__ phi, const T* __restrict__ phi_lo,
-                            double* partials) {
+                            double* partials, Scalars* S, int init) {
   ScalarView<T> F{phi, P.nx, P.ny, P.nz, P.zper};
   const T hih = (T)(0.5 * P.inv_h);
   const T c_a = (T)(3.0 / (2.0 * 1.4142135623730951));
   const T he = (T)(0.5 * P.eps), q = (T)(0.25 / P.eps);
+  const int lanes = row_lanes(P.nx), row0 = (blockIdx.x * kBlock + threadIdx.x) / lanes;
   double sphi = 0.0, sarea = 0.0;
   if constexpr (std::is_same<T, float>::value) {
     // The penalty multipliers use the small differences V - V0 and A - A0,
@@ -115,9 +138,9 @@ __global__ void k_reduce_va(PhaseParams P, const T* __restrict__ phi, const T* _
     // density c_A (eps/2 |grad phi|^2 + (phi^2 - 1)^2 / (4 eps)) from the
     // raw central differences, the constant factors folded into two pairs
     const FF agf{P.ag_hi, P.ag_lo}, awf{P.aw_hi, P.aw_lo};
-    for (int row = blockIdx.x; row < P.ny * P.nz; row += gridDim.x) {
-     const int j = row % P.ny, k = row / P.ny;
-     for (int i = threadIdx.x; i < P.nx; i += blockDim.x) {
+    for (int row = row0; row < P.ny * P.nz; row += gridDim.x * kBlock / lanes) {
+     const int k = row / P.ny, j = row - k * P.ny;
+     for (int i = threadIdx.x & (lanes - 1); i < P.nx; i += lanes) {
       const long long t = lin(i, j, k, P.nx, P.ny);
       const FF f{phi[t], phi_lo[t]};
       auto diff = [&](int i1, int j1, int k1, int i0, int j0, int k0) {
@@ -139,9 +162,9 @@ __global__ void k_reduce_va(PhaseParams P, const T* __restrict__ phi, const T* _
     sphi = (double)cp.hi + (double)cp.lo;
     sarea = (double)ca.hi + (double)ca.lo;
   } else {
-    for (int row = blockIdx.x; row < P.ny * P.nz; row += gridDim.x) {
-     const int j = row % P.ny, k = row / P.ny;
-     for (int i = threadIdx.x; i < P.nx; i += blockDim.x) {
+    for (int row = row0; row < P.ny * P.nz; row += gridDim.x * kBlock / lanes) {
+     const int k = row / P.ny, j = row - k * P.ny;
+     for (int i = threadIdx.x & (lanes - 1); i < P.nx; i += lanes) {
       const long long t = lin(i, j, k, P.nx, P.ny);
       const double f = phi[t];
       const double gx = (F(i + 1, j, k) - F(i - 1, j, k)) * hih;
@@ -153,40 +176,8 @@ __global__ void k_reduce_va(PhaseParams P, const T* __restrict__ phi, const T* _
      }
     }
   }
-  sphi = block_sum(sphi);
-  sarea = block_sum(sarea);
-  if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = sphi;
-    partials[2 * blockIdx.x + 1] = sarea;
-  }
-}
-
-// Fixed-order total of the partials; sets V, A and the multipliers
-// lambda_V = K_V (V - V0), gamma_A = K_A (A - A0) 3 eps / (2 sqrt 2).
-__global__ void k_va_finalize(const double* partials, int nblocks, long long ncells, Scalars* S,
-                              int init) {
-  pdl_begin();
-  double sp = 0.0, sa = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-    sp += partials[2 * b];
-    sa += partials[2 * b + 1];
-  }
-  sp = block_sum(sp);
-  sa = block_sum(sa);
-  if (threadIdx.x == 0) {
-    const double V = 0.5 * S->h3 * ((double)ncells - sp);
-    const double A = S->h3 * sa;
-    S->V = V;
-    S->A = A;
-    if (init) {
-      S->V0 = V;
-      S->A0 = A;
-    }
-    S->lambda_v = S->k_vol * (V - S->V0);
-    S->gamma_a = S->k_area * (A - S->A0) * 3.0 * S->eps / (2.0 * 1.4142135623730951);
-    S->lambda_vf = (float)S->lambda_v;
-    S->gamma_af = (float)S->gamma_a;
-  }
+  __shared__ double buf[2 * kBlock];
+  va_publish(sphi, sarea, buf, partials, (long long)P.nx * P.ny * P.nz, S, init);
 }
 
 // ---------------------------------------------------------------- chemical potential
@@ -1375,6 +1366,10 @@ __global__ void __launch_bounds__(256) k_source_ff4(PhaseParams P, const float* 
   *reinterpret_cast<float4*>(f_lo.p[2] + t) = make_float4(o2l[0], o2l[1], o2l[2], o2l[3]);
 }
 
+// Threads on a row's 4-cell groups in k_reduce_va_ff4.
+__host__ __device__ inline int va4_lanes(int nx) { return nx > 64 ? 32 : (nx > 32 ? 16 : 8); }
+
+
 // Partial sums of sum(phi) and of the area density over 4-cell groups; one
 // (phi, area) pair per block, as k_reduce_va.  Each warp takes whole x rows
 // (row index and plane from one 32-bit division per row), its lanes the
@@ -1385,15 +1380,17 @@ template <bool WITH_G>
 __global__ void __launch_bounds__(256) k_reduce_va_ff4(PhaseParams P, const float* __restrict__ phi,
                                                        const float* __restrict__ phi_lo,
                                                        double* partials, float* __restrict__ g,
-                                                       float* __restrict__ g_lo) {
+                                                       float* __restrict__ g_lo, Scalars* S,
+                                                       int init) {
   pdl_begin();
   const int ng = P.nx >> 2;
   const int rows = P.ny * P.nz;
-  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const int lanes = va4_lanes(P.nx);
   const FF agf{P.ag_hi, P.ag_lo}, awf{P.aw_hi, P.aw_lo};
   CascadeSum cp(0.f), ca(0.f);
-  for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < rows; row += gridDim.x * wpb)
-  for (int gi = lane; gi < ng; gi += 32) {
+  for (int row = (blockIdx.x * kBlock + threadIdx.x) / lanes; row < rows;
+       row += gridDim.x * kBlock / lanes)
+  for (int gi = threadIdx.x & (lanes - 1); gi < ng; gi += lanes) {
     const int k = row / P.ny, j = row - k * P.ny;
     const Geo4 G = geo4(P, 4 * gi, j, k, false);
     const St4 H = load4(phi, G), L = load4(phi_lo, G);
@@ -1428,14 +1425,9 @@ __global__ void __launch_bounds__(256) k_reduce_va_ff4(PhaseParams P, const floa
       *reinterpret_cast<float4*>(g_lo + G.rc + 4 * gi) = make_float4(ol[0], ol[1], ol[2], ol[3]);
     }
   }
-  double sphi = (double)cp.hi + (double)cp.lo;
-  double sarea = (double)ca.hi + (double)ca.lo;
-  sphi = block_sum(sphi);
-  sarea = block_sum(sarea);
-  if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = sphi;
-    partials[2 * blockIdx.x + 1] = sarea;
-  }
+  __shared__ double buf[2 * kBlock];
+  va_publish((double)cp.hi + (double)cp.lo, (double)ca.hi + (double)ca.lo, buf, partials,
+             (long long)P.nx * P.ny * P.nz, S, init);
 }
 
 static bool use4(const PhaseParams& P) { return P.nx % 4 == 0 && P.nx >= 8; }
@@ -1564,27 +1556,26 @@ template <class T>
 bool launch_reduce_va(Ctx& cx, const PhaseParams& P, const T* phi, const T* phi_lo,
                       double* partials, int nblocks, Scalars* S, int init, float* g, float* g_lo) {
   bool with_g = false;
+  const long long rows = (long long)P.ny * P.nz;
   cx.before(VSV_KCLASS_PHASE);
   if constexpr (std::is_same<T, float>::value) {
     if (use4(P)) {
       with_g = g && g_lo;
+      const unsigned blocks = row_blocks(va4_lanes(P.nx), rows, nblocks);
       if (with_g)
-        launch_k(cx, k_reduce_va_ff4<true>, nblocks, kBlock, 0, P, phi, phi_lo, partials, g, g_lo);
+        launch_k(cx, k_reduce_va_ff4<true>, blocks, kBlock, 0, P, phi, phi_lo, partials, g, g_lo, S,
+                 init);
       else
-        launch_k(cx, k_reduce_va_ff4<false>, nblocks, kBlock, 0, P, phi, phi_lo, partials,
-                 (float*)nullptr, (float*)nullptr);
-    } else {
-      k_reduce_va<T><<<nblocks, kBlock, 0, cx.stream>>>(P, phi, phi_lo, partials);
+        launch_k(cx, k_reduce_va_ff4<false>, blocks, kBlock, 0, P, phi, phi_lo, partials,
+                 (float*)nullptr, (float*)nullptr, S, init);
     }
-  } else {
-    k_reduce_va<T><<<nblocks, kBlock, 0, cx.stream>>>(P, phi, phi_lo, partials);
+  }
+  if (!std::is_same<T, float>::value || !use4(P)) {
+    const unsigned blocks = row_blocks(row_lanes(P.nx), rows, nblocks);
+    k_reduce_va<T><<<blocks, kBlock, 0, cx.stream>>>(P, phi, phi_lo, partials, S, init);
   }
   // phi read (two FP32 words, or one FP64); g written (two words)
   cx.after(VSV_KCLASS_PHASE, (with_g ? 16.0 : 8.0) * (double)((long long)P.nx * P.ny * P.nz));
-  cx.before(-1);
-  launch_k(cx, k_va_finalize, 1, kBlock, 0, partials, nblocks, (long long)P.nx * P.ny * P.nz, S,
-           init);
-  cx.after(-1);
   return with_g;
 }
 

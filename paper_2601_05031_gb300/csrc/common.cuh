@@ -286,4 +286,72 @@ struct CascadeSum {
   __device__ __forceinline__ float value() const { return __fadd_rn(hi, lo); }
 };
 
+// Two FP32 numbers in one register pair.  The packed operations round each like
+// the scalar one and take one issue slot for two results (the FP32 units' rate is
+// the same: 37 T operations/s either way), which is what the double-word kernels
+// run short of.  The functions below are the scalar ones above, term for term, on
+// two cells at a time.
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ F2 f2(float a) { return f2(a, a); }
+__device__ __forceinline__ void f2_get(F2 x, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+  F2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F2 neg2(F2 a) {
+  float x, y;
+  f2_get(a, x, y);
+  return f2(-x, -y);
+}
+// Scalar products: a packed one is contracted with an addition that follows it
+// (seen in the error words of a TwoSum), a scalar one is not.
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  float a0, a1, b0, b1;
+  f2_get(a, a0, a1);
+  f2_get(b, b0, b1);
+  return f2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
+}
+__device__ __forceinline__ void two_sum(F2 a, F2 b, F2& s, F2& e) {
+  s = add2(a, b);
+  const F2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+
+struct CascadeSum2 {
+  F2 hi, lo;
+  __device__ __forceinline__ CascadeSum2(F2 a) : hi(a), lo(f2(0.f)) {}
+  __device__ __forceinline__ void add(F2 t) {
+    F2 s, e;
+    two_sum(hi, t, s, e);
+    hi = s;
+    lo = add2(lo, e);
+  }
+  __device__ __forceinline__ void add_scaled(F2 c, F2 x) {
+    const F2 p = mul2(c, x);
+    const F2 pe = fma2(c, x, neg2(p));
+    add(p);
+    lo = add2(lo, pe);
+  }
+};
+
 }  // namespace vsv

@@ -219,33 +219,48 @@ __device__ __forceinline__ float comp4(const float4& v, int o) {
   return o == 0 ? v.x : (o == 1 ? v.y : (o == 2 ? v.z : v.w));
 }
 
-// b - L x at one cell, the same arithmetic as k_defect_dw with every axis
+// b - L x at two cells, the same arithmetic as k_defect_dw with every axis
 // active: hi neighbours by cascaded summation in the order x-, x+, y-, y+,
-// z-, z+, then -6 x_c; lo parts as per-axis pair sums in FP32.
-__device__ __forceinline__ float defect_cell(float xmh, float xph, float ymh, float yph, float zmh,
-                                             float zph, float ch, float xml, float xpl, float yml,
-                                             float ypl, float zml, float zpl, float cl, float b1,
-                                             float b2, bool has_b2, float s, bool has_s,
-                                             float ih_hi, float ih_lo, float dch, float dcl) {
-  CascadeSum lh(xmh);
+// z-, z+, then -6 x_c; lo parts as per-axis pair sums in FP32.  EXTRA: there may be
+// a row source (has_s) or a second diagonal word (dcl).
+template <bool EXTRA>
+__device__ __forceinline__ F2 defect_cells(F2 xmh, F2 xph, F2 ymh, F2 yph, F2 zmh, F2 zph, F2 ch,
+                                           F2 xml, F2 xpl, F2 yml, F2 ypl, F2 zml, F2 zpl, F2 cl,
+                                           F2 b1, F2 b2, bool has_b2, float s, bool has_s,
+                                           float ih_hi, float ih_lo, float dch, float dcl) {
+  CascadeSum2 lh(xmh);
   lh.add(xph);
   lh.add(ymh); lh.add(yph);
   lh.add(zmh); lh.add(zph);
-  float llo = __fadd_rn(__fadd_rn(__fadd_rn(xml, xpl), __fadd_rn(yml, ypl)), __fadd_rn(zml, zpl));
-  lh.add_scaled(-dch, ch);
-  if (dcl != 0.f) lh.add(-dcl * ch);   // adding -0 would change nothing
-  llo = __fmaf_rn(-dch, cl, llo);
-  const float p = __fmul_rn(ih_hi, lh.hi);
-  const float pe = __fmaf_rn(ih_hi, lh.hi, -p);
-  const float rest = __fmaf_rn(ih_hi, __fadd_rn(lh.lo, llo), __fmaf_rn(ih_lo, lh.hi, pe));
-  return defect_combine(b1, b2, has_b2, s, has_s, p, rest);
+  F2 llo = add2(add2(add2(xml, xpl), add2(yml, ypl)), add2(zml, zpl));
+  const F2 md = f2(-dch);
+  lh.add_scaled(md, ch);
+  if (EXTRA && dcl != 0.f) lh.add(mul2(f2(-dcl), ch));   // adding -0 would change nothing
+  llo = fma2(md, cl, llo);
+  const F2 ih = f2(ih_hi);
+  const F2 p = mul2(ih, lh.hi);
+  const F2 pe = fma2(ih, lh.hi, neg2(p));
+  const F2 rest = fma2(ih, add2(lh.lo, llo), fma2(f2(ih_lo), lh.hi, pe));
+  // defect_combine
+  F2 h = b1, lo, d, e;
+  if (EXTRA && has_s) two_sum(b1, f2(s), h, lo);
+  two_sum(h, neg2(p), d, e);
+  lo = EXTRA && has_s ? add2(lo, e) : e;
+  if (has_b2) lo = add2(lo, b2);
+  return add2(d, sub2(lo, rest));
 }
 }  // namespace
 
+// Two cells per instruction (F2): 121 -> 82 instructions a cell.  Then the FP32
+// units, at 0.41 with 24 warps per SM, leave the latency of the loads as the bound.
+// Per launch with three components: 192 x 96 x 80 41.6 -> 38.9 us, 256 x 128 x 128 62.5
+// -> 57 us, 128 x 64 x 64 12.9 -> 11.8 us; 512 x 256 x 256, one component with norms,
+// 165 -> 144 us, of 99 us for its 20 bytes a cell.
+//
 // RAGGED: partial edge tiles; cells past the extent (wrapped copies or zero
 // ghost rows in the staged planes) are skipped.  NORMS: FP64 partial sums of
 // ||r||^2 and ||b||^2 per block (the fixed-cycle solves go without).
-template <int ROWS, bool RAGGED, bool NORMS>
+template <int ROWS, bool RAGGED, bool NORMS, bool EXTRA>
 __global__ void __launch_bounds__(tile::kThreads, ROWS == 1 ? 3 : 2)
 k_defect_tiled(DefGeom G, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R, Comp3<float> BL,
                Comp3<float> OUT, double* partials, Scalars* SC, double* host) {
@@ -309,16 +324,12 @@ k_defect_tiled(DefGeom G, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R, Comp3
   long long gown[ROWS];
 #pragma unroll
   for (int h = 0; h < ROWS; ++h) gown[h] = ((long long)zb * G.ny + jown[h]) * G.nx + x0 + 4 * gx;
-  for (int p = zb, is = zb % kDS; p < ze;
-       ++p, is = (is == kDS - 1) ? 0 : is + 1) {
-    auto sl = [&](float* base, int k) {   // slot of plane p + k, 0 <= k < kDS
-      const int t = is + k;
-      return base + (t >= kDS ? t - kDS : t) * (kDR * kW);
-    };
-    // the step's rhs words and row source, loaded ahead of the barrier so
-    // that their latency overlaps the wait for the staged planes
-    float4 B1s[ROWS], B2s[ROWS];
-    float Ss[ROWS];
+  // the rhs words and row source of a step's plane, loaded a step ahead so that
+  // their latency overlaps a step's arithmetic; with EXTRA's registers that spills,
+  // and they are loaded ahead of the step's barrier
+  float4 B1s[ROWS], B2s[ROWS];
+  float Ss[ROWS];
+  auto load_rhs = [&](int p) {
 #pragma unroll
     for (int h = 0; h < ROWS; ++h) {
       const int j = jown[h];
@@ -326,8 +337,17 @@ k_defect_tiled(DefGeom G, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R, Comp3
       const long long gi = gown[h] + (long long)(p - zb) * plane_n;
       B1s[h] = ok ? *reinterpret_cast<const float4*>(bh + gi) : make_float4(0.f, 0.f, 0.f, 0.f);
       B2s[h] = ok && bl ? *reinterpret_cast<const float4*>(bl + gi) : make_float4(0.f, 0.f, 0.f, 0.f);
-      Ss[h] = ok && S ? S[j + (long long)p * G.ny] : 0.f;
+      Ss[h] = EXTRA && ok && S ? S[j + (long long)p * G.ny] : 0.f;
     }
+  };
+  if (!EXTRA) load_rhs(zb);
+  for (int p = zb, is = zb % kDS; p < ze;
+       ++p, is = (is == kDS - 1) ? 0 : is + 1) {
+    auto sl = [&](float* base, int k) {   // slot of plane p + k, 0 <= k < kDS
+      const int t = is + k;
+      return base + (t >= kDS ? t - kDS : t) * (kDR * kW);
+    };
+    if (EXTRA) load_rhs(p);
     if (p + 3 <= ze) {   // plane p+3 is needed by step p+2
       ds.stage(sl(sH, 3), xh, G, p + 3, false);
       ds.stage(sl(sL, 3), xl, G, p + 3, false);
@@ -344,7 +364,16 @@ k_defect_tiled(DefGeom G, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R, Comp3
       Ph[h] = lds4(sl(sH, 1) + rown[h] * kW + 4 * q);
       Pl[h] = lds4(sl(sL, 1) + rown[h] * kW + 4 * q);
     }
-    float r2 = 0.f, b2 = 0.f;
+    float4 B1c[ROWS], B2c[ROWS];
+    float Sc[ROWS];
+#pragma unroll
+    for (int h = 0; h < ROWS; ++h) {
+      B1c[h] = B1s[h];
+      B2c[h] = B2s[h];
+      Sc[h] = Ss[h];
+    }
+    if (!EXTRA && p + 1 < ze) load_rhs(p + 1);
+    float r2 = 0.f, b2s = 0.f;
 #pragma unroll
     for (int h = 0; h < ROWS; ++h) {
       const int r = rown[h], j = jown[h];
@@ -356,29 +385,39 @@ k_defect_tiled(DefGeom G, Comp3<float> XH, Comp3<float> XL, Rhs3<float> R, Comp3
       const float Lh = rowH[4 * q - 1], Rh = rowH[4 * q + 4];
       const float Ll = rowL[4 * q - 1], Rl = rowL[4 * q + 4];
       const long long gi = gown[h] + (long long)(p - zb) * plane_n;
-      const float4 B1 = B1s[h], B2 = B2s[h];
-      const float s = Ss[h];
+      const float4 B1 = B1c[h], B2 = B2c[h];
+      const float s = Sc[h];
       float res[4];
 #pragma unroll
-      for (int o = 0; o < 4; ++o) {
-        const float xmh = o == 0 ? Lh : comp4(Vh[h], o - 1), xph = o == 3 ? Rh : comp4(Vh[h], o + 1);
-        const float xml = o == 0 ? Ll : comp4(Vl[h], o - 1), xpl = o == 3 ? Rl : comp4(Vl[h], o + 1);
-        const float b1v = beta * comp4(B1, o), b2v = beta * comp4(B2, o);
-        res[o] = defect_cell(xmh, xph, comp4(Uh, o), comp4(Dh, o), comp4(Mh[h], o), comp4(Ph[h], o),
-                             comp4(Vh[h], o), xml, xpl, comp4(Ul, o), comp4(Dl, o), comp4(Ml[h], o),
-                             comp4(Pl[h], o), comp4(Vl[h], o), b1v, b2v, bl != nullptr, s,
-                             S != nullptr, G.ih_hi, G.ih_lo, G.dch, G.dcl);
+      for (int o = 0; o < 4; o += 2) {
+        auto at = [&](const float4& v) { return f2(comp4(v, o), comp4(v, o + 1)); };
+        const F2 xmh = o == 0 ? f2(Lh, Vh[h].x) : f2(Vh[h].y, Vh[h].z);
+        const F2 xph = o == 0 ? f2(Vh[h].y, Vh[h].z) : f2(Vh[h].w, Rh);
+        const F2 xml = o == 0 ? f2(Ll, Vl[h].x) : f2(Vl[h].y, Vl[h].z);
+        const F2 xpl = o == 0 ? f2(Vl[h].y, Vl[h].z) : f2(Vl[h].w, Rl);
+        const F2 b1 = mul2(f2(beta), at(B1)), b2 = mul2(f2(beta), at(B2));
+        const F2 r = defect_cells<EXTRA>(xmh, xph, at(Uh), at(Dh), at(Mh[h]), at(Ph[h]), at(Vh[h]),
+                                         xml, xpl, at(Ul), at(Dl), at(Ml[h]), at(Pl[h]), at(Vl[h]),
+                                         b1, b2, bl != nullptr, s, S != nullptr, G.ih_hi, G.ih_lo,
+                                         G.dch, G.dcl);
+        f2_get(r, res[o], res[o + 1]);
         if (NORMS) {
-          const float bv = b1v + (bl ? b2v : 0.f) + s;
-          r2 = __fmaf_rn(res[o], res[o], r2);
-          b2 = __fmaf_rn(bv, bv, b2);
+          float v1[2], v2[2];
+          f2_get(b1, v1[0], v1[1]);
+          f2_get(b2, v2[0], v2[1]);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const float bv = v1[c] + (bl ? v2[c] : 0.f) + s;
+            r2 = __fmaf_rn(res[o + c], res[o + c], r2);
+            b2s = __fmaf_rn(bv, bv, b2s);
+          }
         }
       }
       *reinterpret_cast<float4*>(out + gi) = make_float4(res[0], res[1], res[2], res[3]);
     }
     if (NORMS) {
       rr += (double)r2;
-      bb += (double)b2;
+      bb += (double)b2s;
     }
   }
   cp_async_wait0();
@@ -426,15 +465,25 @@ int launch_defect_tiled(Ctx& cx, const Level& L, Comp3<float> XH, Comp3<float> X
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem);
       cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     };
-    set(k_defect_tiled<ROWS, false, false>);
-    set(k_defect_tiled<ROWS, true, false>);
-    set(k_defect_tiled<ROWS, false, true>);
-    set(k_defect_tiled<ROWS, true, true>);
+    set(k_defect_tiled<ROWS, false, false, false>);
+    set(k_defect_tiled<ROWS, true, false, false>);
+    set(k_defect_tiled<ROWS, false, true, false>);
+    set(k_defect_tiled<ROWS, true, true, false>);
+    set(k_defect_tiled<ROWS, false, false, true>);
+    set(k_defect_tiled<ROWS, true, false, true>);
+    set(k_defect_tiled<ROWS, false, true, true>);
+    set(k_defect_tiled<ROWS, true, true, true>);
     attr = true;
   }
   dim3 grid(tiles, nz, ncomp);
-  auto kern = aligned ? (partials ? k_defect_tiled<ROWS, false, true> : k_defect_tiled<ROWS, false, false>)
-                      : (partials ? k_defect_tiled<ROWS, true, true> : k_defect_tiled<ROWS, true, false>);
+  auto pick = [&](auto extra) {
+    constexpr bool X = decltype(extra)::value;
+    return aligned ? (partials ? k_defect_tiled<ROWS, false, true, X> : k_defect_tiled<ROWS, false, false, X>)
+                   : (partials ? k_defect_tiled<ROWS, true, true, X> : k_defect_tiled<ROWS, true, false, X>);
+  };
+  bool extra = L.cdl[0] != 0.f;
+  for (int q = 0; q < ncomp; ++q) extra = extra || R.S[q];
+  auto kern = extra ? pick(std::true_type{}) : pick(std::false_type{});
   cx.before(VSV_KCLASS_RESTRICT);
   launch_k(cx, kern, grid, tile::kThreads, Sh::kSmem, G, XH, XL, R, BL, OUT, partials, S, host);
   // x_hi, x_lo, b_hi (, b_lo) read, r written

@@ -517,12 +517,15 @@ bool coarse_plan(const vsv_grid* g, const std::vector<Level>& lv, int m, CoarseC
     // e and r of the two colours, each of half a row's length rounded up
     const long long cols = (long long)((lv[q].n[0] + 1) / 2) * lv[q].n[1], nz = lv[q].n[2];
     off += 4LL * cols * nz;
-    // the shortest runs along z whose threads fit; on a level that runs of 1 to
-    // 8 (FP64: 4) planes do not cover evenly, as many threads as there are
+    // the shortest runs along z whose threads fit (3 and 5 planes on the coarsest
+    // level, where no transfer pairs planes); on a level that runs of 1 to 8 (FP64:
+    // 5) planes do not cover evenly, as many threads as there are
     const long long n = std::min<long long>(kCvThreads, (cols * nz + 31) / 32 * 32);
     long long len = 0;
-    for (long long t = 1; t <= (elem == 4 ? 8 : 4) && !len; t *= 2)
+    for (const long long t : {1, 2, 3, 4, 5, 8}) {
+      if (len || ((t == 3 || t == 5) && q < CC->last) || (t == 8 && elem != 4)) continue;
       if (nz % t == 0 && cols * (nz / t) <= n) len = t;
+    }
     CC->reg[q] = len > 0;
     if (!len) {
       const long long segs = std::max(1LL, n / cols);

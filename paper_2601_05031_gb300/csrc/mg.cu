@@ -586,8 +586,10 @@ __host__ __device__ bool blocked_transfer_ok(const Level& F, const Level& C) {
 // separate arrays of half the row length: a cell's neighbours are all in the
 // other colour's array, at the cell's own index for y and z and at that index
 // and one beside it for x, without unused lanes or bank conflicts.  A thread
-// holds a run of 1, 2, 4 or 8 planes of one column pair in registers (levels
-// that such runs do not cover evenly take a loop over shared memory), and the
+// holds a run of 1, 2, 4 or 8 planes of one column pair in registers, on the
+// coarsest level also 3 or 5 (24 x 12 x 10 cells, 24 sweeps: 22.5 us in runs of
+// 5, 57 us in the loop over shared memory that levels which no such runs cover
+// evenly take), and the
 // boundary rule is resolved once per visit of a level.  A level is worked on
 // by only as many warps as it has runs, on a named barrier of its own (a
 // single warp needs none); the other warps wait for it to come back.
@@ -623,7 +625,8 @@ struct CvLevel {
   int nx, ny, nz, nxh, cols, half;
   int n;                      // threads that work on it
   int runs, len;              // column pairs x runs along z; planes per run
-  bool reg;                   // runs of 1, 2, 4 or 8 planes cover the level evenly
+  bool reg;                   // runs of 1, 2, 4 or 8 planes (3 or 5 too on the coarsest
+                              // level) cover the level evenly
   __device__ __forceinline__ CvLevel(const CoarseCycle& CC, int l) {
     const Level& L = CC.lv[l];
     nx = L.n[0]; ny = L.n[1]; nz = L.n[2];
@@ -923,6 +926,7 @@ __device__ __forceinline__ void cv_visit(const CoarseCycle& CC, int l, const CvL
   const Level& L = CC.lv[l];
   const T h2 = (T)CC.h2[l], c1 = (T)1 - omega;
   const int bar = 1 + l - CC.first;
+  constexpr bool kLast = LEN == 3 || LEN == 5;   // the coarsest level only: from zero, no residual
   CvRegRun<T, LEN> X(L, V, sm);
   X.load_r(V, l == CC.first ? rr : nullptr);
   if (down) {
@@ -930,9 +934,11 @@ __device__ __forceinline__ void cv_visit(const CoarseCycle& CC, int l, const CvL
     for (int q = 0; q < LEN; ++q) X.e[0][q] = X.e[1][q] = (T)0;
   } else {
     X.load_e(V);
-    if (blocked) {
-      X.prolong(V, W, CC.lv[l + 1], sm + W.e);
-      cv_sync(bar, V.n);
+    if constexpr (!kLast) {
+      if (blocked) {
+        X.prolong(V, W, CC.lv[l + 1], sm + W.e);
+        cv_sync(bar, V.n);
+      }
     }
   }
   T w[2][3];   // omega / diagonal: at the run's first plane, inside, at its last
@@ -967,6 +973,7 @@ __device__ __forceinline__ void cv_visit(const CoarseCycle& CC, int l, const CvL
       cv_sync(bar, V.n);
     }
   }
+  if (kLast) return;
   if (resid) {
     if (X.on) {
       const T ih2 = lv_ih2<T>(L);
@@ -1132,6 +1139,8 @@ __device__ __forceinline__ void coarse_vcycle_cta(const CoarseCycle& CC, const T
     else if (V.len == 1) cv_visit<T, 1>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
     else if (V.len == 2) cv_visit<T, 2>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
     else if (V.len == 4) cv_visit<T, 4>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
+    else if (V.len == 3) cv_visit<T, 3>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
+    else if (V.len == 5) cv_visit<T, 5>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
     else cv_visit<T, MAX_LEN>(CC, l, V, W, sm, rr, e_out, sweeps, om, down, rs, blocked);
     if (rs) {
       cv_restrict<T>(CC, l, V, W, sm);

@@ -2577,6 +2577,8 @@ AdjParams adj_params(const vsv_grid* g) {
   P.sigma = g->fe.sigma;
   P.eps = g->fe.eps;
   P.e2 = g->fe.eps * g->fe.eps;
+  P.inv_eps = 1.0 / g->fe.eps;
+  P.ca_eps = 3.0 / (2.0 * std::sqrt(2.0)) / g->fe.eps;
   const double cf1 = 3.0 * std::sqrt(2.0) / (8.0 * std::pow(g->fe.eps, 3));   // C_F per unit kappa
   P.cf2_per_kappa = g->fe.mu_prefactor_half ? cf1 : 2.0 * cf1;
   P.cf2 = P.cf2_per_kappa * g->fe.kappa;

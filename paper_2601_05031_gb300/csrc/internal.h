@@ -463,6 +463,7 @@ struct AdjParams {
   double h, hih, ih2, h3;            // h, 1 / (2h), 1 / h^2, h^3
   int fe_kind;
   double sigma, eps, e2;             // e2 = eps^2
+  double inv_eps, ca_eps;            // 1 / eps, 3 / (2 sqrt 2 eps)
   double cf2, cf2_per_kappa;         // prefactor of the bending mu, and per unit kappa
   double beta;                       // Helfrich tension coefficient sigma c_A / eps
   double inv_eta, mobility, k_vol, k_area;

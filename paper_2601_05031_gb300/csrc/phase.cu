@@ -1369,7 +1369,6 @@ __global__ void __launch_bounds__(256) k_source_ff4(PhaseParams P, const float* 
 // Threads on a row's 4-cell groups in k_reduce_va_ff4.
 __host__ __device__ inline int va4_lanes(int nx) { return nx > 64 ? 32 : (nx > 32 ? 16 : 8); }
 
-
 // Partial sums of sum(phi) and of the area density over 4-cell groups; one
 // (phi, area) pair per block, as k_reduce_va.  Each warp takes whole x rows
 // (row index and plane from one 32-bit division per row), its lanes the

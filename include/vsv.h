@@ -165,8 +165,10 @@ typedef struct {
  *   that level's longest extent, and at least 4); omega_sor <= 0
  * picks the optimal SOR weight for the grid.  variant 0 uses the fastest
  * kernels available for each level (fused single-pass red-black sweeps,
- * tiled transfers and defects where the tile shape allows, the lower levels
- * of a V-cycle in one launch), with partial edge tiles on levels whose
+ * tiled transfers and defects where the tile shape allows, a small level's
+ * pre- or post-smoothing with its transfer in one launch except while a
+ * kernel class is being profiled, the lowest levels of a V-cycle in one
+ * launch), with partial edge tiles on levels whose
  * extents are not multiples of the 128 x 16 tile; 1 forces the reference
  * per-level, per-colour kernels (same arithmetic, bit-identical results; for
  * cross-checks); 2 is 0 without partial tiles (fast kernels on tile-aligned
@@ -338,7 +340,10 @@ vsv_status vsv_stability_limit(const vsv_grid* g, double* dt_max);
  * [nz][ny][nx] arrays of dtype on host or device; x holds the initial guess
  * on entry.  Uses the grid's scratch (it clobbers the grid's flow
  * perturbation of component z; call vsv_set_phi again afterwards to resume
- * time stepping).  cycles_out / relres_out may be NULL. */
+ * time stepping).  cycles_out / relres_out may be NULL.  On the mixed path FP64
+ * rhs and x in memory of the grid's device are read and written in place by
+ * the kernels that split and merge the words; others go through a staging
+ * buffer. */
 vsv_status vsv_solve_poisson(vsv_grid* g, const void* rhs, void* x, int dtype, int on_device,
                              const vsv_bc* bc, double tol, int max_cycles, int* cycles_out,
                              double* relres_out);
@@ -349,7 +354,9 @@ vsv_status vsv_solve_poisson(vsv_grid* g, const void* rhs, void* x, int dtype, i
  * host memory by the copy engine (faster over the host link than a kernel
  * writing mapped memory); with on_device = VSV_HOST_ASYNC that copy runs on
  * the grid's export stream and the call returns at once (valid after
- * vsv_check).  The bits are the same either way; dst needs no alignment. */
+ * vsv_check).  The bits are the same either way; dst needs no alignment.  A
+ * field for memory of the grid's device (aligned to its elements) is written
+ * there by the kernel that forms it, else by a copy. */
 vsv_status vsv_get_field(vsv_grid* g, int field, void* dst, int dtype, int on_device);
 
 /* Replace phi (mu, V, A are recomputed before the next step; V0, A0 and the

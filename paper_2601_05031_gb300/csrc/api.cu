@@ -609,7 +609,7 @@ bool passes_wanted(const vsv_grid* g, const std::vector<Level>& lv, int l, bool 
   if (lv[l].cells() > kPassCells) return false;
   return g->sol.variant == 0 && g->sol.nu1 == 2 && g->sol.nu2 == 2 && x_zero && R.beta == (T)1 &&
          !R.S[0] && !R.S[1] && !R.S[2] && g->cx.prof_class < 0 && l + 1 < (int)lv.size() &&
-         two_sweep_pass_ok(lv[l], lv[l + 1]);
+         two_sweep_pass_ok(lv[l], lv[l + 1]) && two_sweep_pass_ready();
 }
 
 // Largest first level of the one-CTA coarse cycle where the level above it has

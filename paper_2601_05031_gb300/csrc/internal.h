@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <atomic>
 #include <type_traits>
 #include <utility>
 #include <vector>
@@ -90,6 +91,43 @@ void launch_k(const Ctx& cx, void (*kern)(P...), dim3 grid, dim3 block, size_t s
   cfg.attrs = at;
   cfg.numAttrs = (cx.overlap && cx.prof_class < 0) ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+
+// Kernel attributes belong to a device.  once(set) calls set() until it has
+// returned true on the current device, and returns whether it has: a process
+// may have handles on several devices, and calls from several threads (which
+// may then set an attribute twice).  The error of a set() that fails is cleared,
+// one that was pending before is kept.
+class DeviceOnce {
+  static constexpr int kDevices = 64;   // beyond: set on every call
+  std::atomic<bool> done_[kDevices] = {};
+
+ public:
+  template <class F>
+  bool operator()(F&& set) {
+    int dev = -1;
+    const cudaError_t pending = cudaPeekAtLastError();
+    if (cudaGetDevice(&dev) == cudaSuccess) {
+      const bool kept = dev >= 0 && dev < kDevices;
+      if (kept && done_[dev].load(std::memory_order_acquire)) return true;
+      if (set()) {
+        if (kept) done_[dev].store(true, std::memory_order_release);
+        return true;
+      }
+    }
+    if (pending == cudaSuccess) cudaGetLastError();
+    return false;
+  }
+};
+
+// Opt-in of a kernel to `bytes` of dynamic shared memory on the current device,
+// with the largest shared-memory carveout (a preference, which may be ignored).
+template <class K>
+bool allow_smem(K kern, size_t bytes) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+    return false;
+  cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  return true;
 }
 
 // FP64 block reduction (all threads get the block total); blockDim.x must be a
@@ -343,6 +381,7 @@ bool launch_copy_wait_probe(Ctx& cx, const Level& L, Comp3<float> B, Rhs3<float>
 // post-smoothing (prolongation included; the result added to the iterate
 // upd_hi / upd_lo, or stored to OUT, which must not be E)
 bool two_sweep_pass_ok(const Level& F, const Level& C);
+bool two_sweep_pass_ready();   // the current device has granted their shared memory
 void launch_pre_pass(Ctx& cx, const Level& F, const Level& C, Comp3<float> R, Comp3<float> E,
                      Comp3<float> RC, int ncomp, float omega, bool restrict_, int kclass);
 void launch_post_pass(Ctx& cx, const Level& F, const Level& C, Comp3<float> R, Comp3<float> E,

@@ -477,12 +477,6 @@ dim3 pass_grid(const PassGeom& G, int ncomp) {
               (unsigned)ncomp);
 }
 
-template <class K>
-void allow_smem(K kern, size_t bytes) {
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-}
-
 }  // namespace
 
 // Levels the passes serve: every axis active and halved, x periodic in whole
@@ -493,14 +487,18 @@ bool two_sweep_pass_ok(const Level& F, const Level& C) {
          F.n[2] == 2 * C.n[2] && (long long)F.n[0] * F.n[1] < (1LL << 31);
 }
 
+// Every pass kernel's shared memory on the current device; false: the separate
+// kernels do the level's work.
+bool two_sweep_pass_ready() {
+  static DeviceOnce once;
+  return once([] {
+    return allow_smem(k_pre_pass<true>, kSmemRst) && allow_smem(k_pre_pass<false>, kSmemPre) &&
+           allow_smem(k_post_pass<true>, kSmemPost) && allow_smem(k_post_pass<false>, kSmemPost);
+  });
+}
+
 void launch_pre_pass(Ctx& cx, const Level& F, const Level& C, Comp3<float> R, Comp3<float> E,
                      Comp3<float> RC, int ncomp, float omega, bool restrict_, int kclass) {
-  static bool attr = false;
-  if (!attr) {
-    allow_smem(k_pre_pass<true>, kSmemRst);
-    allow_smem(k_pre_pass<false>, kSmemPre);
-    attr = true;
-  }
   const PassGeom G = pass_geom(F, C, omega);
   cx.before(kclass);
   if (restrict_) launch_k(cx, k_pre_pass<true>, pass_grid(G, ncomp), kThr, kSmemRst, G, R, E, RC);
@@ -512,12 +510,6 @@ void launch_pre_pass(Ctx& cx, const Level& F, const Level& C, Comp3<float> R, Co
 void launch_post_pass(Ctx& cx, const Level& F, const Level& C, Comp3<float> R, Comp3<float> E,
                       Comp3<float> EC, Comp3<float> OUT, const Comp3<float>* upd_hi,
                       const Comp3<float>* upd_lo, int ncomp, float omega, int kclass) {
-  static bool attr = false;
-  if (!attr) {
-    allow_smem(k_post_pass<true>, kSmemPost);
-    allow_smem(k_post_pass<false>, kSmemPost);
-    attr = true;
-  }
   const PassGeom G = pass_geom(F, C, omega);
   const Comp3<float> none{{nullptr, nullptr, nullptr}};
   cx.before(kclass);

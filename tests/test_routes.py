@@ -1,0 +1,80 @@
+"""Which kernels the library launches, and what it does on a second device, on
+the CPU: the library's object files linked against a CUDA runtime of the host
+(tests/fake_cuda.cpp) that records launches and keeps each device's kernel
+attributes apart."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    from paper_2601_05031_gb300 import build, vsv
+    build.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libvsv_host.so")
+    objs = [os.path.join(build.OUT_DIR, os.path.basename(s)[:-3] + ".o") for s in build.sources()]
+    if not all(os.path.exists(o) for o in objs):
+        build.build(force=True)
+    inc = os.path.join(os.path.dirname(os.path.dirname(build._nvcc())), "include")
+    # the runtime's symbols bind inside the library, whatever the process has loaded
+    subprocess.run([shutil.which("g++"), "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic",
+                    "-I", inc, os.path.join(HERE, "fake_cuda.cpp"), *objs, "-o", out, "-ldl",
+                    "-lpthread", "-lrt"], check=True)
+    lib = vsv.load(out)
+    lib.fake_name.restype = C.c_char_p
+    lib.fake_refuse.argtypes = [C.c_char_p]
+    return lib
+
+
+def _solve(lib, shape, prec, periodic=(1, 0, 0), device=0, refuse=b"", cycles=1):
+    """The status of one solve of `cycles` cycles and the kernels it launched."""
+    from paper_2601_05031_gb300 import vsv as V
+    nx, ny, nz = shape
+    lib.fake_device(device)
+    lib.fake_refuse(refuse)
+    p = V.VSV_MIXED if prec == "mixed" else V.VSV_FP64
+    need = lib.vsv_workspace_bytes(nx, ny, nz, p)
+    buf = np.zeros(need + 256, dtype=np.uint8)
+    at = (buf.ctypes.data + 255) // 256 * 256
+    g = C.c_void_p()
+    assert lib.vsv_create(C.byref(g), nx, ny, nz, 1.0, p, at, need, None) == V.VSV_OK
+    rhs, x = np.zeros(nx * ny * nz), np.zeros(nx * ny * nz)
+    bc = V.vsv_bc((C.c_int * 3)(*periodic), 0.0)
+    cyc, rr = C.c_int(), C.c_double()
+    lib.fake_clear()
+    st = lib.vsv_solve_poisson(g, rhs.ctypes.data, x.ctypes.data, V.VSV_DTYPE_F64, 1, C.byref(bc), 0.0,
+                               cycles, C.byref(cyc), C.byref(rr))
+    names = [lib.fake_name(i).decode() for i in range(lib.fake_count())]
+    lib.vsv_destroy(g)
+    lib.fake_refuse(b"")
+    lib.fake_device(0)
+    return st, names
+
+
+def _count(names, part):
+    return sum(part in n for n in names)
+
+
+@pytest.mark.parametrize("shape", [(64, 32, 32), (36, 10, 12)])
+def test_passes_opt_in_on_every_device(lib, shape):
+    """The shared-memory limit of the two-sweep passes is an attribute of a
+    kernel on one device: a second device's solve runs the same kernels."""
+    from paper_2601_05031_gb300 import vsv as V
+    for device in (0, 1, 0, 100):
+        st, names = _solve(lib, shape, "mixed", device=device)
+        assert st in (V.VSV_OK, V.VSV_ENOCONV) and _count(names, "k_pre_pass") > 0, device
+
+
+def test_passes_refused_by_the_device_fall_back(lib):
+    """A device that refuses the passes' limit gets the separate kernels."""
+    from paper_2601_05031_gb300 import vsv as V
+    st, names = _solve(lib, (64, 32, 32), "mixed", device=2, refuse=b"k_post_pass")
+    assert st in (V.VSV_OK, V.VSV_ENOCONV)
+    assert _count(names, "k_pre_pass") == 0 and _count(names, "k_post_pass") == 0
+    assert _count(names, "k_rb_sweep") > 0

@@ -1273,12 +1273,14 @@ const void* mapped_host(const void* p) {
 
 // Device memory of the current device with elements of `size` bytes in
 // alignment: a kernel may read or write a field there itself.  Anything else
-// (another device's memory, host pointers, odd offsets) goes by a copy.
+// (another device's memory, host pointers, odd offsets) goes by a copy.  An
+// error that a launch has left pending stays for the caller's check; only the
+// query's own is cleared.
 bool kernel_reachable(const void* p, size_t size) {
   cudaPointerAttributes a;
   int dev = -1;
-  if ((uintptr_t)p % size || cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-      cudaGetDevice(&dev) != cudaSuccess) {
+  if ((uintptr_t)p % size || cudaPeekAtLastError() != cudaSuccess) return false;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

@@ -18,7 +18,7 @@
 namespace {
 int g_dev = 0;
 cudaError_t g_last = cudaSuccess;
-std::string g_refuse;
+std::string g_refuse, g_fail;
 std::map<const void*, std::string> g_names;
 std::map<std::pair<int, const void*>, size_t> g_smem;   // opt-in per (device, kernel)
 std::vector<std::string> g_launches;
@@ -28,6 +28,7 @@ cudaError_t set(cudaError_t e) {
   return e;
 }
 cudaError_t launch(const void* f, size_t smem) {
+  if (!g_fail.empty() && g_names[f].find(g_fail) != std::string::npos) return set(cudaErrorLaunchOutOfResources);
   if (smem > 48 * 1024) {
     const auto it = g_smem.find({g_dev, f});
     if (it == g_smem.end() || it->second < smem) return set(cudaErrorInvalidValue);
@@ -47,6 +48,7 @@ extern "C" {
 // ---- the test's side
 void fake_device(int dev) { g_dev = dev; }
 void fake_refuse(const char* part) { g_refuse = part; }   // kernels whose opt-in fails
+void fake_fail(const char* part) { g_fail = part; }       // kernels whose launch fails
 void fake_clear() { g_launches.clear(); }
 int fake_count() { return (int)g_launches.size(); }
 const char* fake_name(int i) { return g_launches[i].c_str(); }

@@ -28,8 +28,20 @@ def lib(tmp_path_factory):
                     "-lpthread", "-lrt"], check=True)
     lib = vsv.load(out)
     lib.fake_name.restype = C.c_char_p
-    lib.fake_refuse.argtypes = [C.c_char_p]
+    lib.fake_refuse.argtypes = lib.fake_fail.argtypes = [C.c_char_p]
     return lib
+
+
+def _grid(lib, shape, prec):
+    """A handle, and the workspace it lives in."""
+    from paper_2601_05031_gb300 import vsv as V
+    p = V.VSV_MIXED if prec == "mixed" else V.VSV_FP64
+    need = lib.vsv_workspace_bytes(*shape, p)
+    buf = np.zeros(need + 256, dtype=np.uint8)
+    g = C.c_void_p()
+    assert lib.vsv_create(C.byref(g), *shape, 1.0, p, (buf.ctypes.data + 255) // 256 * 256, need,
+                          None) == V.VSV_OK
+    return g, buf
 
 
 def _solve(lib, shape, prec, periodic=(1, 0, 0), device=0, refuse=b"", cycles=1):
@@ -38,12 +50,7 @@ def _solve(lib, shape, prec, periodic=(1, 0, 0), device=0, refuse=b"", cycles=1)
     nx, ny, nz = shape
     lib.fake_device(device)
     lib.fake_refuse(refuse)
-    p = V.VSV_MIXED if prec == "mixed" else V.VSV_FP64
-    need = lib.vsv_workspace_bytes(nx, ny, nz, p)
-    buf = np.zeros(need + 256, dtype=np.uint8)
-    at = (buf.ctypes.data + 255) // 256 * 256
-    g = C.c_void_p()
-    assert lib.vsv_create(C.byref(g), nx, ny, nz, 1.0, p, at, need, None) == V.VSV_OK
+    g, buf = _grid(lib, shape, prec)
     rhs, x = np.zeros(nx * ny * nz), np.zeros(nx * ny * nz)
     bc = V.vsv_bc((C.c_int * 3)(*periodic), 0.0)
     cyc, rr = C.c_int(), C.c_double()
@@ -78,3 +85,24 @@ def test_passes_refused_by_the_device_fall_back(lib):
     assert st in (V.VSV_OK, V.VSV_ENOCONV)
     assert _count(names, "k_pre_pass") == 0 and _count(names, "k_post_pass") == 0
     assert _count(names, "k_rb_sweep") > 0
+
+
+@pytest.mark.parametrize("offset", [0, 4])
+def test_export_reports_the_launch_error_of_its_refresh(lib, offset):
+    """mu of a replaced phi is formed by the export; a kernel of it that fails
+    to launch is reported for any destination, also one that kernels cannot
+    write in place."""
+    from paper_2601_05031_gb300 import vsv as V
+    g, buf = _grid(lib, (16, 8, 8), "mixed")
+    fl, fe = V.vsv_flow_params(V.VSV_COUETTE, 0.0, -0.1, 0.1, 1.0, 0.0), V.vsv_fe_params(
+        V.VSV_CAHN_HILLIARD, 1.0, 0.0, 1.0, 1.0, 0.0, 0.0, 0)
+    assert lib.vsv_set_flow(g, C.byref(fl)) == V.VSV_OK
+    assert lib.vsv_set_free_energy(g, C.byref(fe)) == V.VSV_OK
+    phi, out = np.ones(1024), np.zeros(1026)
+    assert lib.vsv_set_phi(g, phi.ctypes.data, V.VSV_DTYPE_F64, 0) in (V.VSV_OK, V.VSV_ENOCONV)
+    assert lib.vsv_set_field(g, V.VSV_FIELD_PHI, phi.ctypes.data, V.VSV_DTYPE_F64, 1) == V.VSV_OK
+    lib.fake_fail(b"k_mu")
+    st = lib.vsv_get_field(g, V.VSV_FIELD_MU, out.ctypes.data + offset, V.VSV_DTYPE_F64, 1)
+    lib.fake_fail(b"")
+    lib.vsv_destroy(g)
+    assert st == V.VSV_ECUDA

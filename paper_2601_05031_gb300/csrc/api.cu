@@ -636,9 +636,19 @@ bool vcycle(vsv_grid* g, const std::vector<Level>& lv, int l, Comp3<T> X, Rhs3<T
     if (l > 0) {
       Comp3<T> E = X;
       Comp3<T> RR{{(T*)R.B[0], (T*)R.B[1], (T*)R.B[2]}};
+      // One CTA in register runs of planes, or where no runs cover the level in
+      // the loop over shared memory.  On the FP64 path that loop is slower than
+      // k_coarse_solve, and above its 6,144 cells than 48 launches: five cycles at
+      // 36 x 30 x 22 1,700 -> 1,360 us, at 28^3 1,513 -> 1,311, at 56^3 1,903 ->
+      // 1,697, at 44 x 38 x 34 3,155 -> 1,390 (in register runs 796, 1,331 and 1,783
+      // us at 48 x 40 x 24, 36 x 30 x 20 and 44 x 38 x 20; the same without, within
+      // 0.5 %).  FP32: the loop takes 580 us at 36 x 30 x 22 (k_coarse_solve 638),
+      // 764 at 44 x 38 x 34 (1,057), and is level with the launches above
+      // k_coarse_solve's 12,288 cells: 1,253 (1,279) at 60 x 50 x 42, 1,321 (1,270)
+      // at 52 x 50 x 46.
       CoarseCycle CC;
       if (g->sol.variant != 1 && coarse_plan(g, lv, l, &CC, sizeof(T)) &&
-          launch_coarse_vcycle<T>(g->cx, CC, E, RR, ncomp))
+          (sizeof(T) == 4 || CC.reg[l]) && launch_coarse_vcycle<T>(g->cx, CC, E, RR, ncomp))
         return false;
       if (launch_coarse_solve<T>(g->cx, L, E, RR, ncomp, coarsest_sweeps(L, g->sol.coarse_sweeps),
                                  h2))

@@ -106,3 +106,26 @@ def test_export_reports_the_launch_error_of_its_refresh(lib, offset):
     lib.fake_fail(b"")
     lib.vsv_destroy(g)
     assert st == V.VSV_ECUDA
+
+
+@pytest.mark.parametrize("shape,prec,kernel", [
+    ((36, 30, 22), "mixed", "k_coarse_vcycle"),   # 18 x 15 x 11: no runs cover it, FP32
+    ((44, 38, 34), "mixed", "k_coarse_vcycle"),
+    ((36, 30, 22), "fp64", "k_coarse_solve"),     # FP64, up to 6,144 cells
+    ((28, 28, 28), "fp64", "k_coarse_solve"),
+    ((44, 38, 20), "fp64", "k_coarse_vcycle"),    # 22 x 19 x 10: runs of 5 planes
+    ((28, 28, 20), "fp64", "k_coarse_vcycle"),
+    ((44, 38, 34), "fp64", "k_rb_sweep"),         # 7,106 cells: sweeps on every SM
+    ((52, 44, 28), "fp64", "k_rb_sweep"),
+])
+def test_kernel_of_a_lone_coarsest_level(lib, shape, prec, kernel):
+    """A coarsest level below a level with kernels of its own: one CTA holds it
+    in register runs; on the FP64 path, where no runs cover it, the one-CTA
+    solve over shared memory takes it, or above its size launches per colour."""
+    st, names = _solve(lib, shape, prec, cycles=2)
+    for k in ("k_coarse_vcycle", "k_coarse_solve"):
+        assert _count(names, k) == (2 if k == kernel else 0), (k, names)
+    # two cycles: four smoothing sweeps of two colours on the level above, and 24
+    # sweeps of the coarsest where it has launches of its own
+    if prec == "fp64":
+        assert _count(names, "k_rb_sweep") == 2 * (8 + (48 if kernel == "k_rb_sweep" else 0))

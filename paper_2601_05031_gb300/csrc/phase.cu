@@ -680,42 +680,35 @@ __global__ void k_diag_finalize(const double* partials, int nblocks, double* out
 }
 
 // <sigma_xy>(y) = eta <d_y v_x + d_x v_y> over x and z.  The mean of the
-// periodic central difference d_x v_y vanishes term by term, and that of
-// d_y v_x is the central difference of the row means of v_x: one pass that
-// sums v_x over each row of a chunk of planes (double words in cascaded sums),
-// then the differences (308 -> 14 + 4 us at 256 x 128 x 128).
+// periodic central difference d_x v_y vanishes term by term; the differences of
+// v_x are formed and summed in FP64 (sums of v_x would lose to the subtraction of
+// neighbouring rows what v exceeds its differences by).  One block per row and
+// chunk of planes: four FP64 operations a cell.  The call at 256 x 128 x 128: 101 us
+// (differences of sums of v_x in double words 69, of sums in FP64 90 on the FP64
+// path against 100; with d_x v_y summed too, one block a row, 830 and 322).
 template <class T>
-__global__ void k_row_sums(PhaseParams P, const T* __restrict__ vx, const T* __restrict__ vx_lo,
-                           int kchunk, double* sums) {
+__global__ void k_stress_profile(const __grid_constant__ PhaseParams P, const T* __restrict__ vx,
+                                 const T* __restrict__ vx_lo, int kchunk, double scale,
+                                 double* __restrict__ sums) {
   const int j = blockIdx.x, kb = blockIdx.y * kchunk, ke = min(kb + kchunk, P.nz);
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const bool up = j + 1 < P.ny, down = j > 0;
   double s = 0.0;
-  CascadeSum cs(0.f);
   for (int k = kb + (threadIdx.x >> 5); k < ke; k += wpb)
     for (int i = lane; i < P.nx; i += 32) {
       const long long t = lin(i, j, k, P.nx, P.ny);
-      if constexpr (sizeof(T) == 4) {
-        cs.add(vx[t]);
-        cs.add(vx_lo[t]);
-      } else {
-        s += vx[t];
-      }
+      s += (up ? val64(vx, vx_lo, t + P.nx) : P.vwall[1][0]) - (down ? val64(vx, vx_lo, t - P.nx) : P.vwall[0][0]);
     }
-  if constexpr (sizeof(T) == 4) s = (double)cs.hi + (double)cs.lo;
   s = block_sum(s);
-  if (threadIdx.x == 0) sums[(long long)blockIdx.y * P.ny + j] = s;
+  if (threadIdx.x == 0) sums[(long long)blockIdx.y * P.ny + j] = s * scale;
 }
-__global__ void k_stress_profile(PhaseParams P, const double* sums, int chunks, double* out) {
-  const double m = (double)P.nx * (double)P.nz, eta = 1.0 / P.inv_eta;
-  auto row = [&](int j) {
-    if (j < 0) return m * P.vwall[0][0];
-    if (j >= P.ny) return m * P.vwall[1][0];
-    double s = 0.0;
-    for (int c = 0; c < chunks; ++c) s += sums[(long long)c * P.ny + j];
-    return s;
-  };
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < P.ny; j += gridDim.x * blockDim.x)
-    out[j] = eta * ((row(j + 1) - row(j - 1)) * (0.5 * P.inv_h)) / m;
+__global__ void k_profile_total(const double* __restrict__ sums, int ny, int chunks, double scale,
+                                double* __restrict__ out) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= ny) return;
+  double s = 0.0;
+  for (int c = 0; c < chunks; ++c) s += sums[(long long)c * ny + j];
+  out[j] = s * scale;
 }
 
 // ---------------------------------------------------------------- small utilities
@@ -1732,14 +1725,20 @@ void launch_sigma_t(Ctx& cx, const PhaseParams& P, Comp3<T> vel, Comp3<T> vel_lo
 template <class T>
 void launch_stress_profile(Ctx& cx, const PhaseParams& P, const T* vx, const T* vx_lo, double* sums,
                            double* out) {
-  // chunks of planes so that the rows fill the SMs; sums holds ny nz doubles
-  const int chunks = std::max(1, std::min(P.nz, 4 * cx.sms / std::max(1, P.ny)));
+  // chunks of planes so that the rows fill the SMs, of at least 2,048 cells a row
+  // (below, the second launch costs more than it saves); sums holds ny nz doubles
+  const long long cells = (long long)P.nx * P.nz;
+  const int want = (int)std::min<long long>(4 * cx.sms / std::max(1, P.ny), cells / 2048);
+  const int chunks = std::max(1, std::min(P.nz, want));
   const int kchunk = (P.nz + chunks - 1) / chunks, n = (P.nz + kchunk - 1) / kchunk;
+  const double scale = 0.5 * P.inv_h / P.inv_eta / (double)cells;
   cx.before(-1);
-  k_row_sums<T><<<dim3(P.ny, n), kBlock, 0, cx.stream>>>(P, vx, vx_lo, kchunk, sums);
+  k_stress_profile<T><<<dim3(P.ny, n), kBlock, 0, cx.stream>>>(P, vx, vx_lo, kchunk, n > 1 ? 1.0 : scale,
+                                                               n > 1 ? sums : out);
   cx.after(-1);
+  if (n == 1) return;
   cx.before(-1);
-  k_stress_profile<<<(P.ny + 127) / 128, 128, 0, cx.stream>>>(P, sums, n, out);
+  k_profile_total<<<(P.ny + 127) / 128, 128, 0, cx.stream>>>(sums, P.ny, n, scale, out);
   cx.after(-1);
 }
 

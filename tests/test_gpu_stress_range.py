@@ -1,5 +1,7 @@
-"""The in-plane stress over the range of its type, against the FP64 evaluation of
-the exported velocity."""
+"""The in-plane stress over the range of its type and the precision of the stress
+profile: both against the FP64 evaluation of the exported velocity."""
+import math
+
 import numpy as np
 import pytest
 
@@ -95,3 +97,26 @@ def test_stress_field_over_the_range_of_fp64(V, vs, eta):
     # a dozen operations of 2^-53 on differences of values up to max |v|
     tol = 12 * 2.0 ** -53 * eta * 0.5 / h * max(np.abs(a).max() for a in v) * 4
     assert np.max(np.abs(got - ref)) <= tol and np.max(ref) > 100 * tol
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("shape,flow", [((64, 96, 48), "duct"), ((30, 34, 26), "couette"),
+                                        ((128, 128, 96), "duct"), ((32, 8, 256), "duct")])
+def test_stress_profile_as_a_sum_of_fp64_differences(V, shape, flow, prec):
+    nx, ny, nz = shape
+    sim = _state(V, shape, prec, flow, 1.0, 1.3)
+    vx = sim.field(V.VSV_FIELD_VEL_X)
+    prof = sim.stress_profile()
+    sim.close()
+    lo, hi = (-0.3, 0.7) if flow == "couette" else (0.0, 0.0)
+    e = np.concatenate([np.full((nz, 1, nx), lo), vx, np.full((nz, 1, nx), hi)], axis=1)
+    m = nx * nz
+    for j in range(ny):
+        # the mean of the periodic difference d_x v_y vanishes
+        d = e[:, j + 2] - e[:, j]
+        ref = 1.3 * math.fsum(d.ravel()) * 0.5 / m
+        # a thread adds at most m / 256 differences, then come the block's and the
+        # chunks' sums (fewer than 48 additions on any path), each to 2^-53, and
+        # the rounding of a difference
+        tol = (m / 256 + 48) * 2.0 ** -53 * 1.3 * 0.5 * np.mean(np.abs(d))
+        assert abs(prof[j] - ref) <= tol, (j, prof[j], ref, tol)

@@ -459,22 +459,15 @@ int launch_defect_tiled(Ctx& cx, const Level& L, Comp3<float> XH, Comp3<float> X
   G.beta = R.beta;
   G.dch = L.cdh[0];
   G.dcl = L.cdl[0];
-  static bool attr = false;
-  if (!attr) {
-    auto set = [](auto kern) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem);
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    };
-    set(k_defect_tiled<ROWS, false, false, false>);
-    set(k_defect_tiled<ROWS, true, false, false>);
-    set(k_defect_tiled<ROWS, false, true, false>);
-    set(k_defect_tiled<ROWS, true, true, false>);
-    set(k_defect_tiled<ROWS, false, false, true>);
-    set(k_defect_tiled<ROWS, true, false, true>);
-    set(k_defect_tiled<ROWS, false, true, true>);
-    set(k_defect_tiled<ROWS, true, true, true>);
-    attr = true;
-  }
+  static DeviceOnce once;
+  if (!once([] {
+        auto set = [](auto kern) { return allow_smem(kern, Sh::kSmem); };
+        return set(k_defect_tiled<ROWS, false, false, false>) && set(k_defect_tiled<ROWS, true, false, false>) &&
+               set(k_defect_tiled<ROWS, false, true, false>) && set(k_defect_tiled<ROWS, true, true, false>) &&
+               set(k_defect_tiled<ROWS, false, false, true>) && set(k_defect_tiled<ROWS, true, false, true>) &&
+               set(k_defect_tiled<ROWS, false, true, true>) && set(k_defect_tiled<ROWS, true, true, true>);
+      }))
+    return 0;
   dim3 grid(tiles, nz, ncomp);
   auto pick = [&](auto extra) {
     constexpr bool X = decltype(extra)::value;

@@ -726,14 +726,8 @@ template <bool Z, bool HS, bool U, bool RG>
 void launch_variant(dim3 grid, size_t smem, const Ctx& cx, const FusedGeom& G, Comp3<float> A,
                     Comp3<float> B, Rhs3<float> R, Comp3<float> XH, Comp3<float> XL,
                     const FusedMaps& M) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_rbgs_fused<Z, HS, U, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    cudaFuncSetAttribute(k_rbgs_fused<Z, HS, U, RG>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         100);
-    attr_set = true;
-  }
+  static DeviceOnce once;   // a refusal shows in the launch
+  once([&] { return allow_smem(k_rbgs_fused<Z, HS, U, RG>, smem); });
   launch_k(cx, k_rbgs_fused<Z, HS, U, RG>, grid, kThreads, smem, G, A, B, R, XH, XL, M);
 }
 

@@ -326,14 +326,15 @@ bool launch_restrict_tiled(Ctx& cx, const Level& F, const Level& C, Comp3<float>
   G.cnx = C.n[0];
   G.cny = C.n[1];
   const size_t smem = (size_t)kRS * kRR * kW * sizeof(float);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_restrict_tiled<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_restrict_tiled<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_restrict_tiled<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_restrict_tiled<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
+  static DeviceOnce once;
+  if (!once([&] {
+        auto set = [&](auto kern) {
+          return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+        };
+        return set(k_restrict_tiled<false, false>) && set(k_restrict_tiled<true, false>) &&
+               set(k_restrict_tiled<false, true>) && set(k_restrict_tiled<true, true>);
+      }))
+    return false;
   dim3 grid(G.ntx * G.nty, (F.n[2] + G.zchunk - 1) / G.zchunk, ncomp);
   cx.before(VSV_KCLASS_RESTRICT);
   if (R.S[0]) {

@@ -78,6 +78,17 @@ def test_passes_opt_in_on_every_device(lib, shape):
         assert st in (V.VSV_OK, V.VSV_ENOCONV) and _count(names, "k_pre_pass") > 0, device
 
 
+@pytest.mark.parametrize("shape", [(128, 64, 128), (192, 96, 80)])
+def test_tiled_kernels_opt_in_on_every_device(lib, shape):
+    """So do the marching kernels of larger levels (tile-aligned and ragged)."""
+    from paper_2601_05031_gb300 import vsv as V
+    for device in (0, 1, 3):
+        st, names = _solve(lib, shape, "mixed", device=device)
+        assert st in (V.VSV_OK, V.VSV_ENOCONV), device
+        for k in ("k_rbgs_fused", "k_defect_tiled", "k_restrict_tiled"):
+            assert _count(names, k) > 0, (device, k, names)
+
+
 def test_passes_refused_by_the_device_fall_back(lib):
     """A device that refuses the passes' limit gets the separate kernels."""
     from paper_2601_05031_gb300 import vsv as V

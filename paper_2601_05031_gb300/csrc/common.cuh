@@ -93,7 +93,8 @@ __device__ __forceinline__ T mul_t(T a, T b) {
 // of coarse values, already multiplied by their boundary factors, for the
 // (centre plane, centre row), (centre plane, neighbour row), (neighbour
 // plane, centre row) and (neighbour plane, neighbour row).  Every
-// prolongation kernel calls this, so they agree bit for bit.
+// prolongation kernel calls this, or its two parts where cells share the pairs,
+// so they agree bit for bit.
 template <class T>
 __device__ __forceinline__ T prolong_pair(T c, T x) {   // 3/4 c + 1/4 x
   return fma_t((T)0.75, c, mul_t((T)0.25, x));

@@ -668,6 +668,49 @@ __device__ __forceinline__ void cv_runs(const CvLevel& V, F&& f) {
   }
 }
 
+// The prolonged values that a run of column pairs takes from level W (below V,
+// every axis halved): plane() forms those of coarse plane K interpolated in x (the
+// wall factors included) on the even (v[0]) and odd column (v[1]) of the run's own
+// coarse row, and of the row beside it (v[2], v[3]); child() sums the values of a
+// fine plane's own coarse plane (c) and of the one beside it (n).
+template <class T>
+struct CvProlong {
+  int i2, J, xl, xr, jn;
+  T ma, fl, fr, fy;
+  __device__ __forceinline__ CvProlong(const CvRun& R, const CvLevel& W, const Level& C) {
+    ma = -lv_alpha<T>(C);
+    i2 = R.i2;
+    J = R.j >> 1;
+    xl = outer_idx(i2 - 1, W.nx, C.per[0]);
+    xr = outer_idx(i2 + 1, W.nx, C.per[0]);
+    jn = outer_idx(J + ((R.j & 1) ? 1 : -1), W.ny, C.per[1]);
+    fl = xl >= 0 ? (T)1 : ma;
+    fr = xr >= 0 ? (T)1 : ma;
+    fy = jn >= 0 ? (T)1 : ma;
+    if (xl < 0) xl = i2;
+    if (xr < 0) xr = i2;
+    if (jn < 0) jn = J;
+  }
+  __device__ __forceinline__ void plane(const CvLevel& W, const Level& C, const T* we, int K, T v[4]) const {
+    int kk = outer_idx(K, W.nz, C.per[2]);
+    const T fz = kk >= 0 ? (T)1 : ma;
+    if (kk < 0) kk = K < 0 ? 0 : W.nz - 1;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int jj = b ? jn : J;
+      const T f = fz * (b ? fy : (T)1);
+      const T* row = we + (kk * W.ny + jj) * W.nxh;
+      const int sc = (i2 + jj + kk) & 1, hc = sc * W.half, hx = (1 - sc) * W.half;
+      const T n0 = mul_t(f, row[hc + (i2 >> 1)]);
+      v[2 * b] = prolong_pair(n0, mul_t(f * fl, row[((xl ^ i2) & 1 ? hx : hc) + (xl >> 1)]));
+      v[2 * b + 1] = prolong_pair(n0, mul_t(f * fr, row[((xr ^ i2) & 1 ? hx : hc) + (xr >> 1)]));
+    }
+  }
+  static __device__ __forceinline__ T child(const T c[4], const T n[4], int x) {
+    return prolong_sum(c[x], c[2 + x], n[x], n[2 + x]);
+  }
+};
+
 // `sweeps` red-black sweeps (from_zero: e is zero on entry and may hold
 // anything), then (resid) the residual of both colours into the scratch.
 // The neighbour sum, the wall count and the update are those of sum_nb and
@@ -858,37 +901,10 @@ struct CvRegRun {
   // e += P e(W) of the run (every axis halved)
   __device__ __forceinline__ void prolong(const CvLevel& V, const CvLevel& W, const Level& C, const T* we) {
     if (!on) return;
-    const T ma = -lv_alpha<T>(C);
-    const int J = R.j >> 1;
-    int xl = outer_idx(R.i2 - 1, W.nx, C.per[0]), xr = outer_idx(R.i2 + 1, W.nx, C.per[0]);
-    int jn = outer_idx(J + ((R.j & 1) ? 1 : -1), W.ny, C.per[1]);
-    const T fl = xl >= 0 ? (T)1 : ma, fr = xr >= 0 ? (T)1 : ma, fy = jn >= 0 ? (T)1 : ma;
-    if (xl < 0) xl = R.i2;
-    if (xr < 0) xr = R.i2;
-    if (jn < 0) jn = J;
-    // x-interpolated values of coarse plane K (its wall factor included) on the
-    // even and odd column: of the run's own coarse row and of the one beside it
-    auto plane = [&](int K, T v[4]) {
-      int kk = outer_idx(K, W.nz, C.per[2]);
-      const T fz = kk >= 0 ? (T)1 : ma;
-      if (kk < 0) kk = K < 0 ? 0 : W.nz - 1;
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const int jj = b ? jn : J;
-        const T f = fz * (b ? fy : (T)1);
-        const T* row = we + (kk * W.ny + jj) * W.nxh;
-        const int sc = (R.i2 + jj + kk) & 1, hc = sc * W.half, hx = (1 - sc) * W.half;
-        const T n0 = mul_t(f, row[hc + (R.i2 >> 1)]);
-        v[2 * b] = prolong_pair(n0, mul_t(f * fl, row[((xl ^ R.i2) & 1 ? hx : hc) + (xl >> 1)]));
-        v[2 * b + 1] = prolong_pair(n0, mul_t(f * fr, row[((xr ^ R.i2) & 1 ? hx : hc) + (xr >> 1)]));
-      }
-    };
+    const CvProlong<T> I(R, W, C);
+    auto plane = [&](int K, T v[4]) { I.plane(W, C, we, K, v); };
     auto add = [&](int q, const T c[4], const T n[4]) {
-      T v[2];
-#pragma unroll
-      for (int x = 0; x < 2; ++x)
-        v[x] = fma_t((T)0.0625, n[2 + x],
-                     fma_t((T)0.1875, n[x], fma_t((T)0.1875, c[2 + x], mul_t((T)0.5625, c[x]))));
+      const T v[2] = {I.child(c, n, 0), I.child(c, n, 1)};
       const bool par = (R.j + R.k0 + q) & 1;
       e[0][q] += par ? v[1] : v[0];
       e[1][q] += par ? v[0] : v[1];
@@ -1019,38 +1035,11 @@ __device__ __forceinline__ void cv_prolong(const CoarseCycle& CC, int l, const C
   const Level& C = CC.lv[l + 1];
   const T* we = sm + W.e;
   if (blocked_transfer_ok(F, C)) {   // the values of k_prolong_block
-    const T ma = -lv_alpha<T>(C);
     cv_runs(V, [&](const CvRun& R) {
-      const int J = R.j >> 1;
-      int xl = outer_idx(R.i2 - 1, W.nx, C.per[0]), xr = outer_idx(R.i2 + 1, W.nx, C.per[0]);
-      int jn = outer_idx(J + ((R.j & 1) ? 1 : -1), W.ny, C.per[1]);
-      const T fl = xl >= 0 ? (T)1 : ma, fr = xr >= 0 ? (T)1 : ma, fy = jn >= 0 ? (T)1 : ma;
-      if (xl < 0) xl = R.i2;
-      if (xr < 0) xr = R.i2;
-      if (jn < 0) jn = J;
-      // x-interpolated values of coarse plane K (its wall factor included) on
-      // the even (.x) and odd (.y) column: the row's own and the one beside it
-      auto plane = [&](int K, T p[4]) {
-        int kk = outer_idx(K, W.nz, C.per[2]);
-        const T fz = kk >= 0 ? (T)1 : ma;
-        if (kk < 0) kk = K < 0 ? 0 : W.nz - 1;
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          const int jj = b ? jn : J;
-          const T f = fz * (b ? fy : (T)1);
-          const T* row = we + (kk * W.ny + jj) * W.nxh;
-          const int sc = (R.i2 + jj + kk) & 1, hc = sc * W.half, hx = (1 - sc) * W.half;
-          const T n0 = mul_t(f, row[hc + (R.i2 >> 1)]);
-          p[2 * b] = prolong_pair(n0, mul_t(f * fl, row[((xl ^ R.i2) & 1 ? hx : hc) + (xl >> 1)]));
-          p[2 * b + 1] = prolong_pair(n0, mul_t(f * fr, row[((xr ^ R.i2) & 1 ? hx : hc) + (xr >> 1)]));
-        }
-      };
+      const CvProlong<T> I(R, W, C);
+      auto plane = [&](int K, T v[4]) { I.plane(W, C, we, K, v); };
       auto add = [&](int k, const T c[4], const T n[4]) {
-        T v[2];
-#pragma unroll
-        for (int x = 0; x < 2; ++x)
-          v[x] = fma_t((T)0.0625, n[2 + x],
-                       fma_t((T)0.1875, n[x], fma_t((T)0.1875, c[2 + x], mul_t((T)0.5625, c[x]))));
+        const T v[2] = {I.child(c, n, 0), I.child(c, n, 1)};
         T* e = sm + V.e + (k * V.ny + R.j) * V.nxh + R.i2;
         const int par = (R.j + k) & 1;   // the even column's colour
         e[par * V.half] += v[0];

@@ -34,7 +34,7 @@
 // the fused sweeps and tiled transfers, which large levels therefore keep.
 //
 // Arithmetic: rb updates, residuals and prolongation go through nb_term /
-// relax / resid_value / prolong_value's terms with the sums in the order of
+// relax / resid_value / prolong_pair / prolong_sum with the sums in the order of
 // the per-colour kernels, so the results are theirs bit for bit.
 #include <algorithm>
 
@@ -375,12 +375,7 @@ k_post_pass(const __grid_constant__ PassGeom G, Comp3<float> R, Comp3<float> E, 
       const int g8 = 8 * (I.off / 4 - I.row * kG);
       const float* p00 = P + (K * kCRows + J) * kPW + g8;
       const int dj = (I.j & 1) ? kPW : -kPW, dk = (k & 1) ? kCRows * kPW : -kCRows * kPW;
-      auto up = [&](float v, float c, float y, float z, float q) {
-        float acc = mul_t(0.5625f, c);
-        acc = fma_t(0.1875f, y, acc);
-        acc = fma_t(0.1875f, z, acc);
-        return v + fma_t(0.0625f, q, acc);
-      };
+      auto up = [](float v, float c, float y, float z, float q) { return v + prolong_sum(c, y, z, q); };
       auto up4 = [&](float4 v, const float* p) {
         const float4 c = l4(p), y = l4(p + dj), z = l4(p + dk), q = l4(p + dj + dk);
         return make_float4(up(v.x, c.x, y.x, z.x, q.x), up(v.y, c.y, y.y, z.y, q.y),

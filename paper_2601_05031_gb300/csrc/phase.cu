@@ -1819,7 +1819,6 @@ void launch_fill(Ctx& cx, double* x, long long n, double v) {
   template void launch_mu<T>(Ctx&, const PhaseParams&, const T*, T*, T*, const Scalars*);         \
   template void launch_source<T>(Ctx&, const PhaseParams&, const T*, const T*, Comp3<T>,          \
                                  Comp3<T>);                                                       \
-  template void launch_velocity<T>(Ctx&, const PhaseParams&, Comp3<T>, const T*, int, T*);        \
   template void launch_diag<T>(Ctx&, const PhaseParams&, const T*, const T*, const T*, const T*,  \
                                Comp3<T>, Comp3<T>, Comp3<T>, Comp3<T>, Comp3<T>, Comp3<T>,        \
                                Comp3<const double>, Comp3<const double>, double*, int, double*);  \
@@ -1832,6 +1831,8 @@ void launch_fill(Ctx& cx, double* x, long long n, double v) {
 VSV_INST(float)
 VSV_INST(double)
 #undef VSV_INST
+// (the mixed path's velocity is launch_velocity_dw's)
+template void launch_velocity<double>(Ctx&, const PhaseParams&, Comp3<double>, const double*, int, double*);
 template void launch_convert<float, double>(Ctx&, const float*, double*, long long);
 template void launch_convert<double, float>(Ctx&, const double*, float*, long long);
 template void launch_convert<float, float>(Ctx&, const float*, float*, long long);

@@ -140,3 +140,20 @@ def test_kernel_of_a_lone_coarsest_level(lib, shape, prec, kernel):
     # sweeps of the coarsest where it has launches of its own
     if prec == "fp64":
         assert _count(names, "k_rb_sweep") == 2 * (8 + (48 if kernel == "k_rb_sweep" else 0))
+
+
+# kernel counts of one cycle: (pre-smoothing with, without the restriction; post-
+# smoothing with, without the update; one-CTA cycle)
+@pytest.mark.parametrize("shape,periodic,counts", [
+    ((64, 32, 32), (1, 0, 0), (2, 0, 1, 1, 1)),      # 64 x 32 x 32, 32 x 16 x 16; the cycle from 1,024 cells
+    ((128, 64, 16), (1, 0, 1), (2, 0, 1, 1, 1)),     # 2^17 cells: the pass restricts; the cycle from 2,048
+    ((128, 48, 24), (1, 0, 0), (2, 1, 1, 2, 1)),     # above: the tiled restriction; a pass at 2,304 cells
+    ((128, 64, 32), (1, 0, 0), (2, 1, 1, 2, 1)),     # 2^18 cells
+    ((160, 64, 32), (1, 0, 0), (2, 0, 0, 2, 1)),     # above: fused sweeps on the finest level
+    ((64, 32, 32), (0, 0, 0), (0, 0, 0, 0, 1)),      # walls in x: no passes
+])
+def test_passes_run_where_their_sizes_say(lib, shape, periodic, counts):
+    st, names = _solve(lib, shape, "mixed", periodic=periodic)
+    got = tuple(_count(names, k) for k in ("k_pre_passILb1", "k_pre_passILb0", "k_post_passILb1",
+                                           "k_post_passILb0", "k_coarse_vcycleIf"))
+    assert got == counts, names

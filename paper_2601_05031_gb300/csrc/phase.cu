@@ -626,8 +626,9 @@ __device__ __forceinline__ FF shear_dw(FF ap, FF am, FF bp, FF bm, float& tail) 
 // rounding that leaves open (one in 2^15), whose shears cancel by more than about
 // 2^20 or are out of the operations' range (zeros, infinities, NaN, results near
 // FP32's ends), and those beside a wall, whose velocity has 53 bits, take the
-// FP64 evaluation.  The export at 256 x 128 x 128, velocity included: 169 us (in FP64
-// throughout, as on the FP64 path, 345).
+// FP64 evaluation.  83 us at 256 x 128 x 128 (in FP32 double words throughout, with
+// neither the range nor the last bits, 87); the export with its velocity 169 us, on
+// the FP64 path 345.
 __global__ void k_sigma_t_dw(const __grid_constant__ PhaseParams P, const __grid_constant__ Comp3<float> vel,
                              const __grid_constant__ Comp3<float> vel_lo, double f, FF fm, int fe,
                              float* __restrict__ out) {
@@ -683,9 +684,9 @@ __global__ void k_diag_finalize(const double* partials, int nblocks, double* out
 // periodic central difference d_x v_y vanishes term by term; the differences of
 // v_x are formed and summed in FP64 (sums of v_x would lose to the subtraction of
 // neighbouring rows what v exceeds its differences by).  One block per row and
-// chunk of planes: four FP64 operations a cell.  The call at 256 x 128 x 128: 101 us
-// (differences of sums of v_x in double words 69, of sums in FP64 90 on the FP64
-// path against 100; with d_x v_y summed too, one block a row, 830 and 322).
+// chunk of planes: four FP64 operations a cell.  256 x 128 x 128: 45 + 3 us
+// (sums of v_x in FP32 double words 13 + 4); the call 101 us (69), on the FP64 path
+// 100 (sums of v_x 90); with d_x v_y summed too, one block a row, 830 and 322.
 template <class T>
 __global__ void k_stress_profile(const __grid_constant__ PhaseParams P, const T* __restrict__ vx,
                                  const T* __restrict__ vx_lo, int kchunk, double scale,

@@ -681,7 +681,8 @@ __global__ void k_diag_finalize(const double* partials, int nblocks, double* out
 }
 
 // <sigma_xy>(y) = eta <d_y v_x + d_x v_y> over x and z.  The mean of the
-// periodic central difference d_x v_y vanishes term by term; the differences of
+// periodic central difference d_x v_y vanishes term by term, so v_y is not read (a
+// NaN in it alone shows in the diagnostics, not here); the differences of
 // v_x are formed and summed in FP64 (sums of v_x would lose to the subtraction of
 // neighbouring rows what v exceeds its differences by).  One block per row and
 // chunk of planes: four FP64 operations a cell.  256 x 128 x 128: 45 + 3 us
